@@ -6,6 +6,7 @@
 //   sparse: index(pop) = (b * Q + pop) * E^3 + l,     b = block id from the
 //           virtual block map, l = lx + E (ly + E lz)
 #include "d3q19.cuh"
+#include "exact.cuh"
 #include "grid.h"
 
 namespace lbm {
@@ -33,77 +34,130 @@ static LevelDev level_dev(const Level& L) {
   return d;
 }
 
-// Storage base / stride of a virtual-box voxel; false if no storage exists.
-__device__ __forceinline__ bool locate(const LevelDev& d, int x, int y, int z, int64_t& base,
+// Storage base / stride of the virtual-box voxel with linear id v; false if
+// no storage exists.  DENSE needs no coordinates.
+template <bool DENSE>
+__device__ __forceinline__ bool locate(const LevelDev& d, int64_t v, int64_t& base,
                                        int64_t& stride, uint8_t& flag) {
-  if (d.E == 0) {
-    const int64_t v = x + (int64_t)d.nx * (y + (int64_t)d.ny * z);
+  if constexpr (DENSE) {
     base = v;
     stride = d.N;
     flag = d.flags ? d.flags[v] : (uint8_t)0;
     return true;
   }
-  const int E = d.E;
-  const int bx = x / E, by = y / E, bz = z / E;
-  const int b = d.bmap[bx + d.nbx * (by + d.nby * bz)];
+  int x, y, z;
+  if (v <= 0xffffffffLL) {
+    const uint32_t w = (uint32_t)v, row = w / (uint32_t)d.nx;
+    x = (int)(w - row * (uint32_t)d.nx);
+    z = (int)(row / (uint32_t)d.ny);
+    y = (int)(row - (uint32_t)z * (uint32_t)d.ny);
+  } else {
+    const int64_t row = v / d.nx;
+    x = (int)(v - row * d.nx);
+    z = (int)(row / d.ny);
+    y = (int)(row - (int64_t)z * d.ny);
+  }
+  const int e = d.E == 8 ? 3 : 2, M = d.E - 1;
+  const int b = d.bmap[(x >> e) + d.nbx * ((y >> e) + d.nby * (z >> e))];
   if (b < 0) return false;
-  const int l = (x - bx * E) + E * ((y - by * E) + E * (z - bz * E));
-  const int64_t E3 = (int64_t)E * E * E;
-  base = (int64_t)b * Q * E3 + l;
-  stride = E3;
-  flag = d.flags[(int64_t)b * E3 + l];
+  const int l = (x & M) + (((y & M) + ((z & M) << e)) << e);
+  stride = (int64_t)1 << (3 * e);
+  base = (int64_t)b * Q * stride + l;
+  flag = d.flags[(int64_t)b * stride + l];
   return true;
 }
 
+// FP64 forms, for values outside the windows of the exact ones.
 template <int S>
-__global__ void k_init_eq(LevelDev d, void* f, const double* rho, const double* u) {
+__device__ __noinline__ void init_wide(typename Codec<S>::T* out, int64_t stride, double r, double ux,
+                                       double uy, double uz) {
+#pragma unroll
+  for (int i = 0; i < Q; ++i) out[i * stride] = Codec<S>::from_double(feq_d(i, r, ux, uy, uz), i);
+}
+
+template <int S>
+__device__ __noinline__ void sums_wide(const typename Codec<S>::T* in, int64_t stride, double r[4]) {
+  double m = 0, x = 0, y = 0, z = 0;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const double fi = Codec<S>::abs_d(in[i * stride], i);
+    m += fi;
+    if (cx(i)) x += cx(i) * fi;
+    if (cy(i)) y += cy(i) * fi;
+    if (cz(i)) z += cz(i) * fi;
+  }
+  r[0] = m;
+  r[1] = x;
+  r[2] = y;
+  r[3] = z;
+}
+
+// Stored values as floats (FP32: f, 16-bit: s = f - w).
+template <int S>
+__device__ __forceinline__ void load_raw(const typename Codec<S>::T* in, int64_t stride, float v[Q]) {
+  static_for<Q>([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    if constexpr (S == S_F32) v[i] = in[i * stride];
+    else v[i] = Codec<S>::template load<i>(in[i * stride]);
+  });
+}
+
+// Initial state, moments and conservation sums.  In FP64 they were bound by
+// that pipe (29 us per operation and voxel at 256^3: some 190, 125 and 68 of
+// them); with the exact sums and pairs of floats they move DRAM traffic.
+// Measured on GB300, 256^3 FP32, init + moments + conservation: 10.49 ms ->
+// 1.09 ms (DRAM floor 0.73 ms).
+template <int S, bool DENSE>
+__global__ void __launch_bounds__(256) k_init_eq(LevelDev d, void* f, const double* __restrict__ rho,
+                                                 const double* __restrict__ u) {
   using T = typename Codec<S>::T;
   const int64_t n = (int64_t)d.nx * d.ny * d.nz;
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
-    const int x = (int)(v % d.nx);
-    const int y = (int)((v / d.nx) % d.ny);
-    const int z = (int)(v / ((int64_t)d.nx * d.ny));
     int64_t base, stride;
     uint8_t fl;
-    if (!locate(d, x, y, z, base, stride, fl)) continue;
+    if (!locate<DENSE>(d, v, base, stride, fl)) continue;
     if (!type_updated(flag_type(fl))) continue;
     const double r = rho ? rho[v] : 1.0;
     const double ux = u ? u[v] : 0.0, uy = u ? u[n + v] : 0.0, uz = u ? u[2 * n + v] : 0.0;
-    T* out = (T*)f;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) out[base + i * stride] = Codec<S>::from_double(feq_d(i, r, ux, uy, uz), i);
+    T* out = (T*)f + base;
+    EqPair q;
+    bool sure = q.set(r, ux, uy, uz);
+    if (sure)
+      q.all([&](auto ic, DD e) {
+        constexpr int i = decltype(ic)::value;
+        out[i * stride] = eq_store<S>(i, e, sure);
+      });
+    if (!sure) init_wide<S>(out, stride, r, ux, uy, uz);
   }
 }
 
-template <int S>
-__global__ void k_moments(LevelDev d, const void* f, double* rho, double* u) {
+template <int S, bool DENSE>
+__global__ void __launch_bounds__(256) k_moments(LevelDev d, const void* f, double* __restrict__ rho,
+                                                 double* __restrict__ u) {
   using T = typename Codec<S>::T;
   const int64_t n = (int64_t)d.nx * d.ny * d.nz;
   const double nan = __longlong_as_double(0x7ff8000000000000LL);
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
-    const int x = (int)(v % d.nx);
-    const int y = (int)((v / d.nx) % d.ny);
-    const int z = (int)(v / ((int64_t)d.nx * d.ny));
     int64_t base, stride;
     uint8_t fl;
     double r = nan, ux = nan, uy = nan, uz = nan;
-    if (locate(d, x, y, z, base, stride, fl) && type_updated(flag_type(fl))) {
-      const T* in = (const T*)f;
-      double m = 0, jx = 0, jy = 0, jz = 0;
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        const double fi = Codec<S>::abs_d(in[base + i * stride], i);
-        m += fi;
-        jx += cx(i) * fi;
-        jy += cy(i) * fi;
-        jz += cz(i) * fi;
+    if (locate<DENSE>(d, v, base, stride, fl) && type_updated(flag_type(fl))) {
+      const T* in = (const T*)f + base;
+      float g[Q];
+      load_raw<S>(in, stride, g);
+      FixSum<S> q;
+      if (q.set(g)) {
+        fix_moments<S>(q, r, ux, uy, uz);
+      } else {
+        double w[4];
+        sums_wide<S>(in, stride, w);
+        r = w[0];
+        ux = w[1] / r;
+        uy = w[2] / r;
+        uz = w[3] / r;
       }
-      r = m;
-      ux = jx / m;
-      uy = jy / m;
-      uz = jz / m;
     }
     if (rho) rho[v] = r;
     if (u) {
@@ -114,19 +168,16 @@ __global__ void k_moments(LevelDev d, const void* f, double* rho, double* u) {
   }
 }
 
-template <int S>
+template <int S, bool DENSE>
 __global__ void k_decode(LevelDev d, const void* f, double* dst) {
   using T = typename Codec<S>::T;
   const int64_t n = (int64_t)d.nx * d.ny * d.nz;
   const double nan = __longlong_as_double(0x7ff8000000000000LL);
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
-    const int x = (int)(v % d.nx);
-    const int y = (int)((v / d.nx) % d.ny);
-    const int z = (int)(v / ((int64_t)d.nx * d.ny));
     int64_t base, stride;
     uint8_t fl;
-    const bool ok = locate(d, x, y, z, base, stride, fl) && type_updated(flag_type(fl));
+    const bool ok = locate<DENSE>(d, v, base, stride, fl) && type_updated(flag_type(fl));
     const T* in = (const T*)f;
 #pragma unroll
     for (int i = 0; i < Q; ++i)
@@ -136,7 +187,10 @@ __global__ void k_decode(LevelDev d, const void* f, double* dst) {
 
 // ---------------------------------------------------------------- reduction
 // Pass 1: every CTA reduces a fixed, grid-strided set of slots to 4 doubles
-// (warp shuffles, then shared memory) and writes them to partials[cta].
+// (per thread an exact 64-bit fixed-point sum and, for voxels outside its
+// window, an FP64 one; then warp shuffles and shared memory) and writes them
+// to partials[cta].  A thread adds at most N / 311,296 voxels below 2^46
+// units each: no overflow.
 // Pass 2: one CTA adds the partials in a fixed order.  The result does not
 // depend on scheduling, so repeated calls give bit-identical sums.
 constexpr int RED_THREADS = 256;
@@ -154,29 +208,31 @@ __global__ void __launch_bounds__(RED_THREADS) k_cons_partial(LevelDev d, const 
   using T = typename Codec<S>::T;
   const T* in = (const T*)f;
   double acc[4] = {0, 0, 0, 0};
-  const int64_t E3 = d.E ? (int64_t)d.E * d.E * d.E : 1;
+  int64_t fix[4] = {0, 0, 0, 0};
+  const int e = d.E == 0 ? 0 : (d.E == 8 ? 9 : 6);  // log2 of a block's voxels
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < d.N;
        s += (int64_t)gridDim.x * blockDim.x) {
     const uint8_t fl = d.flags ? d.flags[s] : (uint8_t)0;
     if (!type_updated(flag_type(fl))) continue;
-    int64_t base, stride;
-    if (d.E == 0) {
-      base = s;
-      stride = d.N;
+    const int64_t stride = e == 0 ? d.N : (int64_t)1 << e;
+    const T* p = in + (e == 0 ? s : (s >> e) * Q * stride + (s & (stride - 1)));
+    float g[Q];
+    load_raw<S>(p, stride, g);
+    FixSum<S> q;
+    if (q.set(g)) {
+      fix[0] += q.m;
+      fix[1] += q.x;
+      fix[2] += q.y;
+      fix[3] += q.z;
     } else {
-      const int64_t b = s / E3;
-      base = b * Q * E3 + (s - b * E3);
-      stride = E3;
-    }
+      double w[4];
+      sums_wide<S>(p, stride, w);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const double fi = Codec<S>::abs_d(in[base + i * stride], i);
-      acc[0] += fi;
-      if (cx(i)) acc[1] += cx(i) * fi;
-      if (cy(i)) acc[2] += cy(i) * fi;
-      if (cz(i)) acc[3] += cz(i) * fi;
+      for (int k = 0; k < 4; ++k) acc[k] += w[k];
     }
   }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) acc[k] += (double)fix[k] * (1.0 / (double)FixSum<S>::ONE);
   __shared__ double sh[RED_THREADS / 32][4];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
@@ -221,15 +277,33 @@ static unsigned grid_for(int64_t n, int threads) {
   return (unsigned)b;
 }
 
+template <int S>
+static void launch_k_init_eq(const LevelDev& d, unsigned nb, cudaStream_t s, void* f, const double* rho,
+                             const double* u) {
+  if (d.E == 0) k_init_eq<S, true><<<nb, 256, 0, s>>>(d, f, rho, u);
+  else k_init_eq<S, false><<<nb, 256, 0, s>>>(d, f, rho, u);
+}
+template <int S>
+static void launch_k_moments(const LevelDev& d, unsigned nb, cudaStream_t s, const void* f, double* rho,
+                             double* u) {
+  if (d.E == 0) k_moments<S, true><<<nb, 256, 0, s>>>(d, f, rho, u);
+  else k_moments<S, false><<<nb, 256, 0, s>>>(d, f, rho, u);
+}
+template <int S>
+static void launch_k_decode(const LevelDev& d, unsigned nb, cudaStream_t s, const void* f, double* dst) {
+  if (d.E == 0) k_decode<S, true><<<nb, 256, 0, s>>>(d, f, dst);
+  else k_decode<S, false><<<nb, 256, 0, s>>>(d, f, dst);
+}
+
 lbm_status launch_init_equilibrium(Grid& g, Level& L, const double* rho, const double* u,
                                    cudaStream_t s) {
   const LevelDev d = level_dev(L);
   const int64_t n = (int64_t)L.nx * L.ny * L.nz;
   const unsigned nb = grid_for(n, 256);
   switch (g.phys.storage) {
-    case S_F32: k_init_eq<S_F32><<<nb, 256, 0, s>>>(d, L.f[L.cur], rho, u); break;
-    case S_F16: k_init_eq<S_F16><<<nb, 256, 0, s>>>(d, L.f[L.cur], rho, u); break;
-    default: k_init_eq<S_BF16><<<nb, 256, 0, s>>>(d, L.f[L.cur], rho, u); break;
+    case S_F32: launch_k_init_eq<S_F32>(d, nb, s, L.f[L.cur], rho, u); break;
+    case S_F16: launch_k_init_eq<S_F16>(d, nb, s, L.f[L.cur], rho, u); break;
+    default: launch_k_init_eq<S_BF16>(d, nb, s, L.f[L.cur], rho, u); break;
   }
   LBM_CUDA(cudaGetLastError());
   return LBM_OK;
@@ -240,9 +314,9 @@ lbm_status launch_moments(Grid& g, Level& L, double* rho, double* u, cudaStream_
   const int64_t n = (int64_t)L.nx * L.ny * L.nz;
   const unsigned nb = grid_for(n, 256);
   switch (g.phys.storage) {
-    case S_F32: k_moments<S_F32><<<nb, 256, 0, s>>>(d, L.f[L.cur], rho, u); break;
-    case S_F16: k_moments<S_F16><<<nb, 256, 0, s>>>(d, L.f[L.cur], rho, u); break;
-    default: k_moments<S_BF16><<<nb, 256, 0, s>>>(d, L.f[L.cur], rho, u); break;
+    case S_F32: launch_k_moments<S_F32>(d, nb, s, L.f[L.cur], rho, u); break;
+    case S_F16: launch_k_moments<S_F16>(d, nb, s, L.f[L.cur], rho, u); break;
+    default: launch_k_moments<S_BF16>(d, nb, s, L.f[L.cur], rho, u); break;
   }
   LBM_CUDA(cudaGetLastError());
   return LBM_OK;
@@ -253,9 +327,9 @@ lbm_status launch_decode_f64(Grid& g, Level& L, double* dst, cudaStream_t s) {
   const int64_t n = (int64_t)L.nx * L.ny * L.nz;
   const unsigned nb = grid_for(n, 256);
   switch (g.phys.storage) {
-    case S_F32: k_decode<S_F32><<<nb, 256, 0, s>>>(d, L.f[L.cur], dst); break;
-    case S_F16: k_decode<S_F16><<<nb, 256, 0, s>>>(d, L.f[L.cur], dst); break;
-    default: k_decode<S_BF16><<<nb, 256, 0, s>>>(d, L.f[L.cur], dst); break;
+    case S_F32: launch_k_decode<S_F32>(d, nb, s, L.f[L.cur], dst); break;
+    case S_F16: launch_k_decode<S_F16>(d, nb, s, L.f[L.cur], dst); break;
+    default: launch_k_decode<S_BF16>(d, nb, s, L.f[L.cur], dst); break;
   }
   LBM_CUDA(cudaGetLastError());
   return LBM_OK;
