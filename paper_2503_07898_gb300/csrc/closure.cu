@@ -18,6 +18,7 @@
 
 #include "closure.cuh"
 #include "d3q19.cuh"
+#include "exact.cuh"
 #include "grid.h"
 
 namespace lbm {
@@ -334,32 +335,71 @@ __global__ void __launch_bounds__(256) k_reduce(const float* __restrict__ part, 
 }
 
 // Column statistics (mean, standard deviation) of features and targets.
-__global__ void k_stats(const float* X, const float* T, int64_t n, float* stats) {
-  const int c = blockIdx.x;  // 0..16 (16 = target)
-  __shared__ double s1[256], s2[256];
-  double a = 0.0, b = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-    const double v = c < MLP_IN ? X[i * MLP_IN + c] : T[i];
-    a += v;
-    b += v * v;
-  }
-  s1[threadIdx.x] = a;
-  s2[threadIdx.x] = b;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) {
-      s1[threadIdx.x] += s1[threadIdx.x + s];
-      s2[threadIdx.x] += s2[threadIdx.x + s];
+// A CTA takes rows of 64 (16 lanes per row, one column each, so X is read
+// coalesced) and sums v - k and (v - k)^2 as pairs of floats, k = the column's
+// first value: the variance does not cancel against a large mean, which the
+// FP64 sums of v and v^2 did, on 17 CTAs.  Bound by DRAM (68 bytes per sample).
+constexpr int STAT_CTAS = 304;
+__global__ void __launch_bounds__(256) k_stats(const float* __restrict__ X,
+                                               const float* __restrict__ T, int64_t n,
+                                               double* __restrict__ part) {
+  __shared__ double sh[2][16][17];
+  __shared__ double st[2][256];
+  const int c = threadIdx.x & 15, r = threadIdx.x >> 4;
+  DD s1 = {0.f, 0.f}, s2 = {0.f, 0.f}, t1 = {0.f, 0.f}, t2 = {0.f, 0.f};
+  auto take = [](DD& a, DD& b, float v, float k) {
+    const DD d = two_sum(v, -k);
+    dd_acc(a, d);
+    const DD q = two_prod(d.h, d.h);
+    dd_acc(b, {q.h, fmaf(2.f * d.h, d.l, q.l)});
+  };
+  const float kx = X[c], kt = T[0];
+  for (int64_t i0 = (int64_t)blockIdx.x * 64; i0 < n; i0 += (int64_t)gridDim.x * 64) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t i = i0 + 16 * u + r;
+      if (i < n) take(s1, s2, X[i * MLP_IN + c], kx);
     }
-    __syncthreads();
+    if (threadIdx.x < 64 && i0 + threadIdx.x < n) take(t1, t2, T[i0 + threadIdx.x], kt);
+  }
+  sh[0][r][c] = (double)s1.h + s1.l;
+  sh[1][r][c] = (double)s2.h + s2.l;
+  st[0][threadIdx.x] = (double)t1.h + t1.l;
+  st[1][threadIdx.x] = (double)t2.h + t2.l;
+  __syncthreads();
+  if (threadIdx.x < 34) {
+    const int k = threadIdx.x / 17, j = threadIdx.x - 17 * k;
+    double a = 0.0;
+    if (j < MLP_IN)
+      for (int q = 0; q < 16; ++q) a += sh[k][q][j];
+    else
+      for (int q = 0; q < 64; ++q) a += st[k][q];
+    part[(int64_t)blockIdx.x * 34 + threadIdx.x] = a;
+  }
+}
+
+// One warp per column adds the CTAs' sums in a fixed order.
+__global__ void __launch_bounds__(32) k_stats_final(const float* X, const float* T, int64_t n,
+                                                    const double* __restrict__ part, int G,
+                                                    float* stats) {
+  const int c = blockIdx.x;  // 0..16 (16 = target)
+  double a = 0.0, b = 0.0;
+  for (int g = threadIdx.x; g < G; g += 32) {
+    a += part[(int64_t)g * 34 + c];
+    b += part[(int64_t)g * 34 + 17 + c];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
   }
   if (threadIdx.x == 0) {
-    const double mean = s1[0] / (double)n;
-    double var = s2[0] / (double)n - mean * mean;
+    const double d = a / (double)n, mean = (double)(c < MLP_IN ? X[c] : T[0]) + d;
+    double var = b / (double)n - d * d;
     double sd = var > 0 ? sqrt(var) : 0.0;
     // constant column (the tau feature of a one-level set): a deviation below
-    // 1e-6 of the mean's magnitude is rounding noise of the FP64 sums, and as
-    // a scale it would blow up the folded first layer
+    // 1e-6 of the mean's magnitude is rounding noise, and as a scale it would
+    // blow up the folded first layer
     if (!(sd > 1e-30) || !(sd > 1e-6 * fabs(mean))) sd = 1.0;
     const int im = c < MLP_IN ? c : 2 * MLP_IN, is = c < MLP_IN ? MLP_IN + c : 2 * MLP_IN + 1;
     stats[im] = (float)mean;
@@ -401,120 +441,219 @@ struct DsArgs {
   float* den;    // nc
 };
 
+// The kernels below formed their sums, products and quotients in FP64 (some
+// 230 operations per fine voxel and 350 per coarse one at two per SM and
+// clock); as exact sums and pairs of floats (exact.cuh; results rounded to
+// FP32, as before) they cost FP32 operations only.  Measured on GB300, 256^3
+// FP32, r = 2, dataset + statistics + 20 training steps: 11.2 ms -> 2.0 ms.
+
+// rho and j of a fine voxel outside the exact sums' window, from FP64.
+__device__ __noinline__ void filter_wide(const float v[Q], bool shifted, DD* out) {
+  double m = 0, x = 0, y = 0, z = 0;
+  for (int i = 0; i < Q; ++i) {
+    const double f = shifted ? wd(i) + (double)v[i] : (double)v[i];
+    m += f;
+    x += cx(i) * f;
+    y += cy(i) * f;
+    z += cz(i) * f;
+  }
+  const double d[4] = {m, x, y, z};
+  for (int k = 0; k < 4; ++k) {
+    out[k].h = (float)d[k];
+    out[k].l = (float)(d[k] - (double)out[k].h);
+  }
+}
+
+// mean of n values whose sum is s, minus w, to FP32
+__device__ __forceinline__ float mean_minus(DD s, float n, DD inv_n, float wh, float wl) {
+  const DD q = two_prod(n, wh), d = two_sum(s.h, -q.h);
+  const DD t = quick_sum(d.h, add_rn(d.l, sub_rn(s.l, fmaf(n, wl, q.l))));
+  return dd_mul(t, inv_n).h;
+}
+
+// One thread per coarse voxel.  The sums of the populations collect every
+// rounding error (dd_acc); rho and j of each fine voxel are exact.
 template <int S>
-__global__ void k_ds_filter(DsArgs a) {
+__global__ void __launch_bounds__(128) k_ds_filter(DsArgs a) {
   using T = typename Codec<S>::T;
   const int64_t nc = (int64_t)a.cx_ * a.cy_ * a.cz_;
   const int64_t X = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (X >= nc) return;
-  const int Xx = (int)(X % a.cx_), Xy = (int)((X / a.cx_) % a.cy_), Xz = (int)(X / ((int64_t)a.cx_ * a.cy_));
-  const T* f = (const T*)a.f;
-  double sp[Q], m[10];
-  for (int i = 0; i < Q; ++i) sp[i] = 0;
-  for (int k = 0; k < 10; ++k) m[k] = 0;
-  for (int dz = 0; dz < a.r; ++dz)
-    for (int dy = 0; dy < a.r; ++dy)
-      for (int dx = 0; dx < a.r; ++dx) {
-        const int64_t v = (Xx * a.r + dx) + (int64_t)a.nx * ((Xy * a.r + dy) + (int64_t)a.ny * (Xz * a.r + dz));
-        double rho = 0, jx = 0, jy = 0, jz = 0;
+  const int row = (int)(X / a.cx_), Xx = (int)(X - (int64_t)row * a.cx_), Xz = row / a.cy_, Xy = row - Xz * a.cy_;
+  DD sp[Q], m[10];
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-          const double fi = Codec<S>::abs_d(f[(int64_t)i * a.N + v], i);
-          sp[i] += fi - wd(i);
-          rho += fi;
-          jx += cx(i) * fi;
-          jy += cy(i) * fi;
-          jz += cz(i) * fi;
-        }
-        m[0] += rho;
-        m[1] += jx;
-        m[2] += jy;
-        m[3] += jz;
-        m[4] += jx * jx / rho;
-        m[5] += jy * jy / rho;
-        m[6] += jz * jz / rho;
-        m[7] += jx * jy / rho;
-        m[8] += jx * jz / rho;
-        m[9] += jy * jz / rho;
+  for (int i = 0; i < Q; ++i) sp[i] = {0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < 10; ++k) m[k] = {0.f, 0.f};
+#pragma unroll 1
+  for (int dz = 0; dz < a.r; ++dz)
+#pragma unroll 1
+    for (int dy = 0; dy < a.r; ++dy) {
+      const T* f = (const T*)a.f + (Xx * a.r + (int64_t)a.nx * ((Xy * a.r + dy) + (int64_t)a.ny * (Xz * a.r + dz)));
+#pragma unroll 1
+      for (int dx = 0; dx < a.r; ++dx, ++f) {
+        float v[Q];
+        static_for<Q>([&](auto ic) {
+          constexpr int i = decltype(ic)::value;
+          if constexpr (S == S_F32) v[i] = f[(int64_t)i * a.N];
+          else v[i] = Codec<S>::template load<i>(f[(int64_t)i * a.N]);
+        });
+#pragma unroll
+        for (int i = 0; i < Q; ++i) dd_acc(sp[i], v[i]);
+        FixSum<S> q;
+        DD c[4];
+        if (!q.set(v, c)) filter_wide(v, S != S_F32, c);
+        const DD inv = dd_inv(c[0]);
+        const DD ux = dd_mul(c[1], inv), uy = dd_mul(c[2], inv), uz = dd_mul(c[3], inv);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) dd_acc(m[k], c[k]);
+        dd_acc(m[4], dd_mul(c[1], ux));
+        dd_acc(m[5], dd_mul(c[2], uy));
+        dd_acc(m[6], dd_mul(c[3], uz));
+        dd_acc(m[7], dd_mul(c[1], uy));
+        dd_acc(m[8], dd_mul(c[1], uz));
+        dd_acc(m[9], dd_mul(c[2], uz));
       }
-  const double inv = 1.0 / ((double)a.r * a.r * a.r);
-  for (int i = 0; i < Q; ++i) a.sbar[(int64_t)i * nc + X] = (float)(sp[i] * inv);
-  for (int k = 0; k < 10; ++k) a.mom[(int64_t)k * nc + X] = (float)(m[k] * inv);
+    }
+  const float n = (float)((int64_t)a.r * a.r * a.r);
+  const DD inv = dd_inv({n, 0.f});
+  static_for<Q>([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    constexpr float wh = S == S_F32 ? (float)wd(i) : 0.f;
+    constexpr float wl = S == S_F32 ? (float)(wd(i) - (double)(float)wd(i)) : 0.f;
+    a.sbar[(int64_t)i * nc + X] = mean_minus(sp[i], n, inv, wh, wl);
+  });
+#pragma unroll
+  for (int k = 0; k < 10; ++k) a.mom[(int64_t)k * nc + X] = mean_minus(m[k], n, inv, 0.f, 0.f);
 }
 
+// Index of a coarse voxel with every coordinate in [-1, c].
 __device__ __forceinline__ int64_t cidx(const DsArgs& a, int x, int y, int z) {
-  x = (x + a.cx_) % a.cx_;
-  y = (y + a.cy_) % a.cy_;
-  z = (z + a.cz_) % a.cz_;
-  return x + (int64_t)a.cx_ * (y + (int64_t)a.cy_ * z);
+  auto wrap = [](int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); };
+  return wrap(x, a.cx_) + (int64_t)a.cx_ * (wrap(y, a.cy_) + (int64_t)a.cy_ * wrap(z, a.cz_));
+}
+// Coordinates of the calling thread's coarse voxel; false past the end.
+__device__ __forceinline__ bool cvoxel(const DsArgs& a, int64_t& X, int& x, int& y, int& z) {
+  X = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (X >= (int64_t)a.cx_ * a.cy_ * a.cz_) return false;
+  const int row = (int)(X / a.cx_);
+  x = (int)(X - (int64_t)row * a.cx_);
+  z = row / a.cy_;
+  y = row - z * a.cy_;
+  return true;
 }
 
-__global__ void k_ds_features(DsArgs a, float tau, float* feats) {
+__global__ void __launch_bounds__(128) k_ds_features(DsArgs a, float tau, float* feats) {
   const int64_t nc = (int64_t)a.cx_ * a.cy_ * a.cz_;
-  const int64_t X = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (X >= nc) return;
-  const int x = (int)(X % a.cx_), y = (int)((X / a.cx_) % a.cy_), z = (int)(X / ((int64_t)a.cx_ * a.cy_));
+  int64_t X;
+  int x, y, z;
+  if (!cvoxel(a, X, x, y, z)) return;
   float s[Q];
 #pragma unroll
   for (int i = 0; i < Q; ++i) s[i] = a.sbar[(int64_t)i * nc + cidx(a, x - cx(i), y - cy(i), z - cz(i))];
   float xf[MLP_IN];
   closure_features(s, tau, xf);
-  for (int k = 0; k < MLP_IN; ++k) feats[X * MLP_IN + k] = xf[k];
+  float* o = feats + X * MLP_IN;
+  if (((uintptr_t)feats & 15) == 0) {  // uniform: the rows are 64 bytes
+#pragma unroll
+    for (int k = 0; k < MLP_IN; k += 4)
+      *reinterpret_cast<float4*>(o + k) = make_float4(xf[k], xf[k + 1], xf[k + 2], xf[k + 3]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < MLP_IN; ++k) o[k] = xf[k];
+  }
 }
 
-__global__ void k_ds_numden(DsArgs a) {
+// Numerator and denominator of the least-squares eddy viscosity.
+__global__ void __launch_bounds__(128) k_ds_numden(DsArgs a) {
   const int64_t nc = (int64_t)a.cx_ * a.cy_ * a.cz_;
-  const int64_t X = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (X >= nc) return;
-  const int x = (int)(X % a.cx_), y = (int)((X / a.cx_) % a.cy_), z = (int)(X / ((int64_t)a.cx_ * a.cy_));
-  auto ub = [&](int b, int xx, int yy, int zz) {
-    const int64_t i = cidx(a, xx, yy, zz);
-    return (double)a.mom[(int64_t)(1 + b) * nc + i] / (double)a.mom[i];
-  };
-  double g[3][3];  // g[a][b] = d u_b / d x_a
-  for (int b = 0; b < 3; ++b) {
-    g[0][b] = 0.5 * (ub(b, x + 1, y, z) - ub(b, x - 1, y, z));
-    g[1][b] = 0.5 * (ub(b, x, y + 1, z) - ub(b, x, y - 1, z));
-    g[2][b] = 0.5 * (ub(b, x, y, z + 1) - ub(b, x, y, z - 1));
-  }
-  const double rb = a.mom[X];
-  const double u[3] = {a.mom[1 * nc + X] / rb, a.mom[2 * nc + X] / rb, a.mom[3 * nc + X] / rb};
-  const int pa[6] = {0, 1, 2, 0, 0, 1}, pb[6] = {0, 1, 2, 1, 2, 2};
-  double t[3][3];
-  for (int k = 0; k < 6; ++k) {
-    const double v = (double)a.mom[(int64_t)(4 + k) * nc + X] - rb * u[pa[k]] * u[pb[k]];
-    t[pa[k]][pb[k]] = v;
-    t[pb[k]][pa[k]] = v;
-  }
-  const double tr = (t[0][0] + t[1][1] + t[2][2]) / 3.0;
-  double num = 0, den = 0;
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) {
-      const double Sij = 0.5 * (g[i][j] + g[j][i]);
-      num += (t[i][j] - (i == j ? tr : 0.0)) * Sij;
-      den += Sij * Sij;
+  int64_t X;
+  int x, y, z;
+  if (!cvoxel(a, X, x, y, z)) return;
+  // j / rho of FP32 values: quotient and remainder
+  auto vel = [&](int64_t i, DD u[3]) {
+    const float r = a.mom[i], w = 1.f / r;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const float j = a.mom[(int64_t)(1 + b) * nc + i], q = mul_rn(j, w);
+      u[b] = quick_sum(q, mul_rn(fmaf(-q, r, j), w));
     }
-  a.num[X] = (float)num;
-  a.den[X] = (float)(2.0 * rb * den);
+  };
+  DD g[3][3];  // g[a][b] = 2 d u_b / d x_a
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    DD p[3], m[3];
+    vel(cidx(a, x + (d == 0), y + (d == 1), z + (d == 2)), p);
+    vel(cidx(a, x - (d == 0), y - (d == 1), z - (d == 2)), m);
+#pragma unroll
+    for (int b = 0; b < 3; ++b) g[d][b] = dd_add(p[b], neg(m[b]));
+  }
+  DD u[3];
+  vel(X, u);
+  // sub-filter stress: mean(j_a j_b / rho) - j_a u_b
+  DD t[6];  // xx yy zz xy xz yz
+  auto stress = [&](int k, int p, int q) {
+    const float j = a.mom[(int64_t)(1 + p) * nc + X];
+    const DD e = two_prod(j, u[q].h);
+    t[k] = dd_add({a.mom[(int64_t)(4 + k) * nc + X], 0.f}, neg(quick_sum(e.h, fmaf(j, u[q].l, e.l))));
+  };
+  stress(0, 0, 0);
+  stress(1, 1, 1);
+  stress(2, 2, 2);
+  stress(3, 0, 1);
+  stress(4, 0, 2);
+  stress(5, 1, 2);
+  const DD third = {0x1.555556p-2f, -0x1.555556p-27f};
+  const DD tr = dd_mul(dd_add(dd_add(t[0], t[1]), t[2]), third);
+  DD num = {0.f, 0.f}, den = {0.f, 0.f};
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {  // S_ii = g_ii / 2
+    const DD s = {0.5f * g[i][i].h, 0.5f * g[i][i].l};
+    num = dd_add(num, dd_mul(dd_add(t[i], neg(tr)), s));
+    den = dd_add(den, dd_mul(s, s));
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {  // 2 S_ij = (g_ij + g_ji) / 2, twice in the sums
+    const int i = k == 2 ? 1 : 0, j = k == 0 ? 1 : 2;
+    const DD e = dd_add(g[i][j], g[j][i]);
+    const DD s2 = {0.5f * e.h, 0.5f * e.l};
+    num = dd_add(num, dd_mul(t[3 + k], s2));
+    const DD q = dd_mul(s2, s2);
+    den = dd_add(den, {0.5f * q.h, 0.5f * q.l});
+  }
+  a.num[X] = num.h;
+  a.den[X] = dd_mul(den, {2.f * a.mom[X], 0.f}).h;
 }
 
-__global__ void k_ds_target(DsArgs a, float tau, float* targets) {
-  const int64_t nc = (int64_t)a.cx_ * a.cy_ * a.cz_;
-  const int64_t X = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (X >= nc) return;
-  const int x = (int)(X % a.cx_), y = (int)((X / a.cx_) % a.cy_), z = (int)(X / ((int64_t)a.cx_ * a.cy_));
-  double n = 0, d = 0;
+__global__ void __launch_bounds__(128) k_ds_target(DsArgs a, float tau, float* targets) {
+  int64_t X;
+  int x, y, z;
+  if (!cvoxel(a, X, x, y, z)) return;
+  DD n = {0.f, 0.f}, d = {0.f, 0.f};
+#pragma unroll
   for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll
     for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
       for (int dx = -1; dx <= 1; ++dx) {
         const int64_t i = cidx(a, x + dx, y + dy, z + dz);
-        n += a.num[i];
-        d += a.den[i];
+        dd_acc(n, a.num[i]);
+        dd_acc(d, a.den[i]);
       }
-  double t = d > 0 ? -3.0 * n / d : 0.0;
-  const double lo = -((double)tau - 0.5) + 1e-3;
-  t = t < lo ? lo : (t > 0.5 ? 0.5 : t);
-  targets[X] = (float)t;
+  n = quick_sum(n.h, n.l);
+  d = quick_sum(d.h, d.l);
+  float t = 0.f;
+  if (d.h > 0.f) {
+    const float lo = (float)(-((double)tau - 0.5) + 1e-3);
+    if (d.h > 1e-30f) {
+      const DD q = dd_mul(n, dd_inv(d)), p = two_prod(-3.f, q.h);
+      t = add_rn(p.h, fmaf(-3.f, q.l, p.l));
+    } else {  // 1 / d would overflow
+      t = (float)(-3.0 * ((double)n.h + n.l) / ((double)d.h + d.l));
+    }
+    t = t < lo ? lo : (t > 0.5f ? 0.5f : t);
+  }
+  targets[X] = t;
 }
 
 }  // namespace lbm
@@ -576,12 +715,15 @@ lbm_status lbm_closure_train(const float* feats, const float* targets, int64_t n
   // and the column statistics
   const int G = minibatch_ctas(batch);
   const size_t n_part = (size_t)G * PART;
-  DevBuf buf((n_part + 2 * PART + 64) * sizeof(float));
+  DevBuf buf((n_part + 2 * PART + 64) * sizeof(float) + STAT_CTAS * 34 * sizeof(double));
   lbm_status st = buf.p ? LBM_OK : fail(LBM_ERR_OOM, "device allocation failed");
   if (!st) {
     float *part = buf.f(), *m = part + n_part, *v = m + PART, *stats = v + PART, *loss = stats + 48;
+    double* spart = reinterpret_cast<double*>(stats + 64);  // an even number of floats from the base
+    const int SG = (int)(n < STAT_CTAS * 64LL ? (n + 63) / 64 : STAT_CTAS);
     cudaMemsetAsync(m, 0, 2 * PART * sizeof(float), s);
-    k_stats<<<MLP_IN + 1, 256, 0, s>>>(feats, targets, n, stats);
+    k_stats<<<SG, 256, 0, s>>>(feats, targets, n, spart);
+    k_stats_final<<<MLP_IN + 1, 32, 0, s>>>(feats, targets, n, spart, SG, stats);
     for (int it = 1; it <= steps; ++it) {
       k_minibatch<<<G, 256, 0, s>>>(theta_io, feats, targets, n, nullptr, seed, (int64_t)(it - 1) * batch,
                                     batch, stats, part);
