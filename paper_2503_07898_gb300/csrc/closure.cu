@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(256) k_reduce(const float* __restrict__ part, 
 // coalesced) and sums v - k and (v - k)^2 as pairs of floats, k = the column's
 // first value: the variance does not cancel against a large mean, which the
 // FP64 sums of v and v^2 did, on 17 CTAs.  Bound by DRAM (68 bytes per sample).
-constexpr int STAT_CTAS = 304;
+constexpr int STAT_CTAS = 1216;  // eight per SM: the chains of dependent additions need the warps
 __global__ void __launch_bounds__(256) k_stats(const float* __restrict__ X,
                                                const float* __restrict__ T, int64_t n,
                                                double* __restrict__ part) {
@@ -378,13 +378,13 @@ __global__ void __launch_bounds__(256) k_stats(const float* __restrict__ X,
   }
 }
 
-// One warp per column adds the CTAs' sums in a fixed order.
-__global__ void __launch_bounds__(32) k_stats_final(const float* X, const float* T, int64_t n,
+// One CTA per column adds the CTAs' sums in a fixed order.
+__global__ void __launch_bounds__(256) k_stats_final(const float* X, const float* T, int64_t n,
                                                     const double* __restrict__ part, int G,
                                                     float* stats) {
   const int c = blockIdx.x;  // 0..16 (16 = target)
   double a = 0.0, b = 0.0;
-  for (int g = threadIdx.x; g < G; g += 32) {
+  for (int g = threadIdx.x; g < G; g += 256) {
     a += part[(int64_t)g * 34 + c];
     b += part[(int64_t)g * 34 + 17 + c];
   }
@@ -393,7 +393,17 @@ __global__ void __launch_bounds__(32) k_stats_final(const float* X, const float*
     a += __shfl_xor_sync(0xffffffffu, a, o);
     b += __shfl_xor_sync(0xffffffffu, b, o);
   }
+  __shared__ double sa[8], sb[8];
+  if ((threadIdx.x & 31) == 0) {
+    sa[threadIdx.x >> 5] = a;
+    sb[threadIdx.x >> 5] = b;
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) {
+      a += sa[w];
+      b += sb[w];
+    }
     const double d = a / (double)n, mean = (double)(c < MLP_IN ? X[c] : T[0]) + d;
     double var = b / (double)n - d * d;
     double sd = var > 0 ? sqrt(var) : 0.0;
@@ -418,13 +428,30 @@ constexpr unsigned REDUCE_CTAS = (P_LOSS + 1 + 31) / 32;
 struct DevBuf {
   void* p = nullptr;
   explicit DevBuf(size_t bytes) {
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    if (bytes && cudaMalloc(&p, bytes) != cudaSuccess) {
       cudaGetLastError();
       p = nullptr;
     }
   }
   ~DevBuf() {
     if (p) cudaFree(p);
+  }
+  float* f() const { return (float*)p; }
+};
+
+// The same from the device's stream-ordered pool (a training call ends with a
+// synchronisation, at which the pool gives the memory back).
+struct StreamBuf {
+  void* p = nullptr;
+  cudaStream_t s;
+  StreamBuf(size_t bytes, cudaStream_t st) : s(st) {
+    if (cudaMallocAsync(&p, bytes, s) != cudaSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
+  }
+  ~StreamBuf() {
+    if (p) cudaFreeAsync(p, s);
   }
   float* f() const { return (float*)p; }
 };
@@ -445,7 +472,7 @@ struct DsArgs {
 // 230 operations per fine voxel and 350 per coarse one at two per SM and
 // clock); as exact sums and pairs of floats (exact.cuh; results rounded to
 // FP32, as before) they cost FP32 operations only.  Measured on GB300, 256^3
-// FP32, r = 2, dataset + statistics + 20 training steps: 11.2 ms -> 2.0 ms.
+// FP32, r = 2, dataset + statistics + 20 training steps: 11.2 ms -> 1.4 ms.
 
 // rho and j of a fine voxel outside the exact sums' window, from FP64.
 __device__ __noinline__ void filter_wide(const float v[Q], bool shifted, DD* out) {
@@ -471,9 +498,11 @@ __device__ __forceinline__ float mean_minus(DD s, float n, DD inv_n, float wh, f
   return dd_mul(t, inv_n).h;
 }
 
-// One thread per coarse voxel.  The sums of the populations collect every
-// rounding error (dd_acc); rho and j of each fine voxel are exact.
-template <int S>
+// One thread per coarse voxel.  rho and j of each fine voxel are exact.  The
+// population sums add the split parts: up to 8^3 upper parts stay below 2^24
+// units and the lower ones round at 2^-34 at worst.  LARGE (r > 8): they
+// collect every rounding error instead (dd_acc).
+template <int S, bool LARGE>
 __global__ void __launch_bounds__(128) k_ds_filter(DsArgs a) {
   using T = typename Codec<S>::T;
   const int64_t nc = (int64_t)a.cx_ * a.cy_ * a.cz_;
@@ -498,21 +527,32 @@ __global__ void __launch_bounds__(128) k_ds_filter(DsArgs a) {
           if constexpr (S == S_F32) v[i] = f[(int64_t)i * a.N];
           else v[i] = Codec<S>::template load<i>(f[(int64_t)i * a.N]);
         });
-#pragma unroll
-        for (int i = 0; i < Q; ++i) dd_acc(sp[i], v[i]);
         FixSum<S> q;
         DD c[4];
-        if (!q.set(v, c)) filter_wide(v, S != S_F32, c);
+        {
+          float h[Q], l[Q];
+          const bool ok = FixSum<S>::split(v, h, l);
+          if (!q.pairs(h, l, ok, c)) filter_wide(v, S != S_F32, c);
+#pragma unroll
+          for (int i = 0; i < Q; ++i) {
+            if constexpr (LARGE) {
+              dd_acc(sp[i], v[i]);
+            } else {
+              sp[i].h = add_rn(sp[i].h, h[i]);
+              sp[i].l = add_rn(sp[i].l, l[i]);
+            }
+          }
+        }
         const DD inv = dd_inv(c[0]);
         const DD ux = dd_mul(c[1], inv), uy = dd_mul(c[2], inv), uz = dd_mul(c[3], inv);
 #pragma unroll
         for (int k = 0; k < 4; ++k) dd_acc(m[k], c[k]);
-        dd_acc(m[4], dd_mul(c[1], ux));
-        dd_acc(m[5], dd_mul(c[2], uy));
-        dd_acc(m[6], dd_mul(c[3], uz));
-        dd_acc(m[7], dd_mul(c[1], uy));
-        dd_acc(m[8], dd_mul(c[1], uz));
-        dd_acc(m[9], dd_mul(c[2], uz));
+        dd_acc(m[4], dd_prod(c[1], ux));
+        dd_acc(m[5], dd_prod(c[2], uy));
+        dd_acc(m[6], dd_prod(c[3], uz));
+        dd_acc(m[7], dd_prod(c[1], uy));
+        dd_acc(m[8], dd_prod(c[1], uz));
+        dd_acc(m[9], dd_prod(c[2], uz));
       }
     }
   const float n = (float)((int64_t)a.r * a.r * a.r);
@@ -521,10 +561,15 @@ __global__ void __launch_bounds__(128) k_ds_filter(DsArgs a) {
     constexpr int i = decltype(ic)::value;
     constexpr float wh = S == S_F32 ? (float)wd(i) : 0.f;
     constexpr float wl = S == S_F32 ? (float)(wd(i) - (double)(float)wd(i)) : 0.f;
-    a.sbar[(int64_t)i * nc + X] = mean_minus(sp[i], n, inv, wh, wl);
+    a.sbar[(int64_t)i * nc + X] = mean_minus(two_sum(sp[i].h, sp[i].l), n, inv, wh, wl);
   });
 #pragma unroll
   for (int k = 0; k < 10; ++k) a.mom[(int64_t)k * nc + X] = mean_minus(m[k], n, inv, 0.f, 0.f);
+}
+
+template <int S> static void ds_filter(const DsArgs& a, unsigned nb, cudaStream_t s) {
+  if (a.r > 8) k_ds_filter<S, true><<<nb, 128, 0, s>>>(a);
+  else k_ds_filter<S, false><<<nb, 128, 0, s>>>(a);
 }
 
 // Index of a coarse voxel with every coordinate in [-1, c].
@@ -715,7 +760,7 @@ lbm_status lbm_closure_train(const float* feats, const float* targets, int64_t n
   // and the column statistics
   const int G = minibatch_ctas(batch);
   const size_t n_part = (size_t)G * PART;
-  DevBuf buf((n_part + 2 * PART + 64) * sizeof(float) + STAT_CTAS * 34 * sizeof(double));
+  StreamBuf buf((n_part + 2 * PART + 64) * sizeof(float) + STAT_CTAS * 34 * sizeof(double), s);
   lbm_status st = buf.p ? LBM_OK : fail(LBM_ERR_OOM, "device allocation failed");
   if (!st) {
     float *part = buf.f(), *m = part + n_part, *v = m + PART, *stats = v + PART, *loss = stats + 48;
@@ -723,7 +768,7 @@ lbm_status lbm_closure_train(const float* feats, const float* targets, int64_t n
     const int SG = (int)(n < STAT_CTAS * 64LL ? (n + 63) / 64 : STAT_CTAS);
     cudaMemsetAsync(m, 0, 2 * PART * sizeof(float), s);
     k_stats<<<SG, 256, 0, s>>>(feats, targets, n, spart);
-    k_stats_final<<<MLP_IN + 1, 32, 0, s>>>(feats, targets, n, spart, SG, stats);
+    k_stats_final<<<MLP_IN + 1, 256, 0, s>>>(feats, targets, n, spart, SG, stats);
     for (int it = 1; it <= steps; ++it) {
       k_minibatch<<<G, 256, 0, s>>>(theta_io, feats, targets, n, nullptr, seed, (int64_t)(it - 1) * batch,
                                     batch, stats, part);
@@ -780,18 +825,25 @@ lbm_status lbm_closure_dataset(lbm_grid* h, int r, double tau_coarse, float* fea
   a.cz_ = L.nz / r;
   a.N = L.n_slots;
   const int64_t nc = (int64_t)a.cx_ * a.cy_ * a.cz_;
-  DevBuf sbar(nc * Q * 4), mom(nc * 10 * 4), num(nc * 4), den(nc * 4);
-  if (!sbar.p || !mom.p || !num.p || !den.p) return fail(LBM_ERR_OOM, "device allocation failed");
-  a.sbar = sbar.f();
-  a.mom = mom.f();
-  a.num = num.f();
-  a.den = den.f();
+  // Scratch: 31 floats per coarse voxel.  The buffer that the next step
+  // overwrites has room for them when r > 1 and holds nothing that is read
+  // before (every voxel of a grid without flags is written by a step).
+  const size_t need = (size_t)nc * (Q + 12) * 4;
+  std::lock_guard<std::mutex> hold(g.spare_mutex);
+  const bool spare = !L.flags_d && need <= L.pop_bytes;
+  DevBuf own(spare ? 0 : need);
+  if (!spare && !own.p) return fail(LBM_ERR_OOM, "device allocation failed");
+  if (spare) g.spare_used = true;
+  a.sbar = spare ? (float*)L.f[L.cur ^ 1] : own.f();
+  a.mom = a.sbar + nc * Q;
+  a.num = a.mom + nc * 10;
+  a.den = a.num + nc;
   cudaStream_t s = g.stream;
   const unsigned nb = (unsigned)((nc + 127) / 128);
   switch (g.phys.storage) {
-    case S_F32: k_ds_filter<S_F32><<<nb, 128, 0, s>>>(a); break;
-    case S_F16: k_ds_filter<S_F16><<<nb, 128, 0, s>>>(a); break;
-    default: k_ds_filter<S_BF16><<<nb, 128, 0, s>>>(a); break;
+    case S_F32: ds_filter<S_F32>(a, nb, s); break;
+    case S_F16: ds_filter<S_F16>(a, nb, s); break;
+    default: ds_filter<S_BF16>(a, nb, s); break;
   }
   k_ds_features<<<nb, 128, 0, s>>>(a, (float)tau_coarse, feats);
   k_ds_numden<<<nb, 128, 0, s>>>(a);

@@ -101,6 +101,11 @@ __host__ __device__ __forceinline__ DD dd_mul(DD a, DD b) {
   const DD p = two_prod(a.h, b.h);
   return quick_sum(p.h, fmaf(a.h, b.l, fmaf(a.l, b.h, p.l)));
 }
+// The same without renormalising, for sums.
+__host__ __device__ __forceinline__ DD dd_prod(DD a, DD b) {
+  const DD p = two_prod(a.h, b.h);
+  return {p.h, fmaf(a.h, b.l, fmaf(a.l, b.h, p.l))};
+}
 // Accumulate x (or a pair) without renormalising: s.l collects the errors.
 __host__ __device__ __forceinline__ void dd_acc(DD& s, float x) {
   const DD t = two_sum(s.h, x);
@@ -156,8 +161,8 @@ template <int S> struct FixSum {
   float rho;           // rho in FP32 (a starting value for its reciprocal)
 
   // v: the stored values as floats (FP32: f; 16-bit: s).  False if a value
-  // is outside the window or rho is not in [1/16, 64).  parts: the sums as
-  // floats, upper and lower (rho, j; without the 1 of 16-bit storage).
+  // is outside the window or rho is not in [1/16, 64).  parts: the sums of
+  // the upper and lower parts (rho, j; without the 1 of 16-bit storage).
   __host__ __device__ __forceinline__ bool set(const float v[Q]) {
     float a[4], b[4];
     const bool ok = parts(v, a, b);
@@ -167,25 +172,20 @@ template <int S> struct FixSum {
     z = fix(a[3], b[3]);
     return ok;
   }
-  // The same sums as pairs of floats: rho, j.
-  __host__ __device__ __forceinline__ bool set(const float v[Q], DD c[4]) {
-    float a[4], b[4];
-    const bool ok = parts(v, a, b);
-    c[0] = two_sum(a[0], b[0]);
-    if (S != S_F32) {
-      const DD s = two_sum(1.f, c[0].h);
-      c[0] = quick_sum(s.h, add_rn(s.l, c[0].l));
-    }
-#pragma unroll
-    for (int k = 1; k < 4; ++k) c[k] = two_sum(a[k], b[k]);
-    return ok;
-  }
   __host__ __device__ __forceinline__ bool parts(const float v[Q], float a[4], float b[4]) {
+    float h[Q], l[Q];
+    const bool ok = split(v, h, l);
+    sums(h, a);
+    sums(l, b);
+    rho = S == S_F32 ? a[0] + b[0] : 1.f + a[0];
+    return ok && rho >= 0.0625f && rho < 64.f;
+  }
+  // The two parts of each value (v = h + l always); whether all are in the window.
+  __host__ __device__ static __forceinline__ bool split(const float v[Q], float h[Q], float l[Q]) {
     constexpr float UP = S == S_F32 ? 768.f : 12.f;  // 1.5 2^23 upper units
     constexpr uint32_t LOW = (S == S_F32 ? 127u - 11u : 127u - 33u) << 23;
     constexpr uint32_t TOP = (S == S_F32 ? 128u : 126u) << 23;
     uint32_t mn = 0xffffffffu, mx = 0u;
-    float h[Q], l[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       if constexpr (S == S_F32) {
@@ -203,9 +203,21 @@ template <int S> struct FixSum {
     bool ok = mx < TOP;
     if constexpr (S == S_F32) ok = ok && mn >= LOW;
     if constexpr (S == S_BF16) ok = ok && mn >= LOW - 1u;
+    return ok;
+  }
+  // From split parts: rho, j as pairs of floats.
+  __host__ __device__ __forceinline__ bool pairs(const float h[Q], const float l[Q], bool ok, DD c[4]) {
+    float a[4], b[4];
     sums(h, a);
     sums(l, b);
     rho = S == S_F32 ? a[0] + b[0] : 1.f + a[0];
+    c[0] = two_sum(a[0], b[0]);
+    if (S != S_F32) {
+      const DD s = two_sum(1.f, c[0].h);
+      c[0] = quick_sum(s.h, add_rn(s.l, c[0].l));
+    }
+#pragma unroll
+    for (int k = 1; k < 4; ++k) c[k] = two_sum(a[k], b[k]);
     return ok && rho >= 0.0625f && rho < 64.f;
   }
 

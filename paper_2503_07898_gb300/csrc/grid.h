@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -134,6 +135,12 @@ struct Grid {
   // step's stream every step
   cudaStream_t grp_hi = nullptr;
   cudaEvent_t grp_fork = nullptr, grp_join = nullptr;
+
+  // dense grids without flags: lbm_closure_dataset works in the buffer that the
+  // next step overwrites (one call at a time); spare_used: that buffer holds
+  // such values, to be cleared should walls be set before the next step
+  std::mutex spare_mutex;
+  bool spare_used = false;
 
   // learned closure (multi-resolution levels >= 1)
   void* closure_d = nullptr;     // ClosureParams on the device
