@@ -87,6 +87,15 @@ template <int N, int I = 0, class F> __device__ __forceinline__ void static_for(
   }
 }
 
+// In a kernel that a chained launch may have made resident early: waits until
+// the kernels before it have completed, then lets the next one become
+// resident (in this order, so at most two of a chain overlap and no kernel
+// starts before the last but one has finished).
+__device__ __forceinline__ void chain() {
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+}
+
 enum Storage { S_F32 = 0, S_F16 = 1, S_BF16 = 2 };
 
 namespace LBM_LNS {

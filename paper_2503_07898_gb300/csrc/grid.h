@@ -155,6 +155,25 @@ struct Grid {
   void dfree(void* p, cudaStream_t s);
 };
 
+// Launch of a step's kernel that may become resident while the kernel before it
+// on the stream drains (programmatic dependent launch): the kernel calls
+// chain() before it touches population data, which waits for everything before it.
+// chained = false: an ordinary launch.
+template <class... P, class... A>
+cudaError_t launch_step(bool chained, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, P(args)...);
+}
+
 // Fork the boundary-group stream from s (*hi receives it) / join it back.
 lbm_status group_fork(Grid& g, cudaStream_t s, cudaStream_t* hi);
 lbm_status group_join(Grid& g, cudaStream_t s);
@@ -163,6 +182,9 @@ lbm_status group_join(Grid& g, cudaStream_t s);
 int prof_begin(Grid& g, cudaStream_t s, const char* name, int64_t units);
 void prof_end(Grid& g, cudaStream_t s, int rec);
 void prof_clear(Grid& g);
+
+// Gives the closure training's idle workspace back (closure.cu).
+void closure_trim(int device);
 
 // Kernel launchers (defined in the .cu files) -------------------------------
 // dense.cu, sparse.cu, fields.cu and multires.cu are built once per lattice, into
