@@ -464,7 +464,9 @@ lbm_status lbm_grid_create_multires(const int finest_dims[3], int n_levels,
 
 lbm_status lbm_grid_destroy(lbm_grid* h) {
   if (!h) return fail(LBM_ERR_INVALID, "grid is NULL");
+  const int device = h->g.device;
   free_grid(h->g);
+  closure_trim(device);
   delete h;
   return LBM_OK;
 }

@@ -81,7 +81,9 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {
 // the batch).
 // What bounds it: a step is 127 MFLOP (B = 4096) spread over 128 CTAs, so the
 // two launches' latency and the chain gather -> layers -> gradient, not a
-// pipe.  Tiles of 32 give one CTA per SM at B = 4096; a thread's 2 x 4
+// pipe.  The launches are chained (each becomes resident while the one before
+// drains), and what another launch of the chain has written is read through
+// L2.  Tiles of 32 give one CTA per SM at B = 4096; a thread's 2 x 4
 // outputs of a layer take 6 16-byte shared loads per 32 FMAs.
 // Measured on GB300, per step at B = 4096: 22 us (the ten separate kernels it
 // replaces, one thread per output with strided global loads: 640 us).
@@ -134,14 +136,51 @@ __global__ void __launch_bounds__(256) k_minibatch(const float* __restrict__ th,
                                                    float* __restrict__ part) {
   __shared__ TrainSmem sm;
   const int tid = threadIdx.x;
-  for (int i = tid; i < MLP_H * MLP_IN; i += 256) sm.w1[(i >> 4) * SW1 + (i & 15)] = th[P_W1 + i];
-  for (int i = tid; i < MLP_H * MLP_H; i += 256) sm.w2[(i >> 6) * SW2 + (i & 63)] = th[P_W2 + i];
-  if (tid < MLP_H) {
-    sm.b1[tid] = th[P_B1 + tid];
-    sm.b2[tid] = th[P_B2 + tid];
-    sm.w3[tid] = th[P_W3 + tid];
+  // gather of a tile: 8 threads per sample, two features each; rows past the
+  // batch take part with zeros and a zero output gradient.  The first tile's
+  // samples do not depend on the step before, so their loads come ahead of
+  // the wait for it; the next tile's go out before this one's arithmetic.
+  float x0, x1, tv;
+  auto gather = [&](int64_t b0) {
+    const int s = tid >> 3, k = (tid & 7) * 2;
+    const int64_t b = b0 + s;
+    x0 = x1 = tv = 0.f;
+    if (b < B) {
+      const int64_t i = idx ? (int64_t)idx[b]
+                            : (int64_t)(splitmix64(seed + (uint64_t)(counter0 + b)) % (uint64_t)n);
+      x0 = X[i * MLP_IN + k];
+      x1 = X[i * MLP_IN + k + 1];
+      if (k == 0) tv = T[i];
+      if (stats) {
+        x0 = (x0 - stats[k]) / stats[MLP_IN + k];
+        x1 = (x1 - stats[k + 1]) / stats[MLP_IN + k + 1];
+        if (k == 0) tv = (tv - stats[2 * MLP_IN]) / stats[2 * MLP_IN + 1];
+      }
+    }
+  };
+  gather((int64_t)blockIdx.x * TT);
+  chain();
+  if (((uintptr_t)th & 15) == 0) {  // uniform
+    const float4 v = __ldcg(reinterpret_cast<const float4*>(th + P_W1 + 4 * tid));
+    float4 w[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) w[q] = __ldcg(reinterpret_cast<const float4*>(th + P_W2 + 4 * (tid + 256 * q)));
+    *reinterpret_cast<float4*>(sm.w1 + (tid >> 2) * SW1 + (tid & 3) * 4) = v;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = tid + 256 * q;
+      *reinterpret_cast<float4*>(sm.w2 + (i >> 4) * SW2 + (i & 15) * 4) = w[q];
+    }
+  } else {
+    for (int i = tid; i < MLP_H * MLP_IN; i += 256) sm.w1[(i >> 4) * SW1 + (i & 15)] = __ldcg(th + P_W1 + i);
+    for (int i = tid; i < MLP_H * MLP_H; i += 256) sm.w2[(i >> 6) * SW2 + (i & 63)] = __ldcg(th + P_W2 + i);
   }
-  if (tid == 0) sm.b3 = th[P_B3];
+  if (tid < MLP_H) {
+    sm.b1[tid] = __ldcg(th + P_B1 + tid);
+    sm.b2[tid] = __ldcg(th + P_B2 + tid);
+    sm.w3[tid] = __ldcg(th + P_W3 + tid);
+  }
+  if (tid == 0) sm.b3 = __ldcg(th + P_B3);
   const int tx = tid & 15, ty = tid >> 4;
   float g2[4][4], g1[4], gv = 0.f;  // W2, W1, and one of b2 / b1 / W3 / b3 / loss
 #pragma unroll
@@ -151,28 +190,13 @@ __global__ void __launch_bounds__(256) k_minibatch(const float* __restrict__ th,
     for (int i = 0; i < 4; ++i) g2[j][i] = 0.f;
   }
   for (int64_t b0 = (int64_t)blockIdx.x * TT; b0 < B; b0 += (int64_t)gridDim.x * TT) {
-    // gather: 8 threads per sample, two features each; rows past the batch
-    // take part with zeros and a zero output gradient
     {
       const int s = tid >> 3, k = (tid & 7) * 2;
-      const int64_t b = b0 + s;
-      float x0 = 0.f, x1 = 0.f, t = 0.f;
-      if (b < B) {
-        const int64_t i = idx ? (int64_t)idx[b]
-                              : (int64_t)(splitmix64(seed + (uint64_t)(counter0 + b)) % (uint64_t)n);
-        x0 = X[i * MLP_IN + k];
-        x1 = X[i * MLP_IN + k + 1];
-        if (k == 0) t = T[i];
-        if (stats) {
-          x0 = (x0 - stats[k]) / stats[MLP_IN + k];
-          x1 = (x1 - stats[k + 1]) / stats[MLP_IN + k + 1];
-          if (k == 0) t = (t - stats[2 * MLP_IN]) / stats[2 * MLP_IN + 1];
-        }
-      }
       sm.x[s * SW1 + k] = x0;
       sm.x[s * SW1 + k + 1] = x1;
-      if (k == 0) sm.t[s] = t;
+      if (k == 0) sm.t[s] = tv;
     }
+    gather(b0 + (int64_t)gridDim.x * TT);
     __syncthreads();
     layer_2x4<MLP_IN>(sm.x, SW1, sm.w1, SW1, sm.b1, 2 * ty, tx, sm.h1);
     __syncthreads();
@@ -311,9 +335,10 @@ __global__ void __launch_bounds__(256) k_reduce(const float* __restrict__ part, 
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane;
   float s = 0.f;
+  chain();
   if (i <= P_LOSS) {
 #pragma unroll 8
-    for (int c = w; c < G; c += 8) s += part[(int64_t)c * PART + i];
+    for (int c = w; c < G; c += 8) s += __ldcg(part + (int64_t)c * PART + i);
   }
   sh[w][lane] = s;
   __syncthreads();
@@ -417,6 +442,20 @@ __global__ void __launch_bounds__(256) k_stats_final(const float* X, const float
   }
 }
 
+// Folds the normalisation into the first and last layers.
+__global__ void __launch_bounds__(MLP_H) k_fold(float* th, const float* __restrict__ sv) {
+  const int j = threadIdx.x;
+  double b = th[P_B1 + j];
+  for (int k = 0; k < MLP_IN; ++k) {
+    const float w = th[P_W1 + j * MLP_IN + k];
+    b -= (double)w * sv[k] / sv[MLP_IN + k];
+    th[P_W1 + j * MLP_IN + k] = w / sv[MLP_IN + k];
+  }
+  th[P_B1 + j] = (float)b;
+  th[P_W3 + j] *= sv[2 * MLP_IN + 1];
+  if (j == 0) th[P_B3] = th[P_B3] * sv[2 * MLP_IN + 1] + sv[2 * MLP_IN];
+}
+
 // CTAs of a minibatch: one per tile of 32 samples, at most two per SM (a CTA
 // then takes several tiles), which bounds the partial buffer to 6.5 MB.
 static int minibatch_ctas(int B) {
@@ -439,19 +478,48 @@ struct DevBuf {
   float* f() const { return (float*)p; }
 };
 
-// The same from the device's stream-ordered pool (a training call ends with a
-// synchronisation, at which the pool gives the memory back).
+// A training call's workspace, from a stream-ordered pool per device that keeps at
+// most 16 MB between calls (a call needs up to 7 MB; mapping them anew cost
+// 150 us of it) and gives them back when a grid is destroyed.
+static cudaMemPool_t work_pool(int device, bool create) {
+  static std::mutex m;
+  static cudaMemPool_t pools[64] = {};
+  if (device < 0 || device >= 64) return nullptr;
+  std::lock_guard<std::mutex> hold(m);
+  if (!pools[device] && create) {
+    cudaMemPoolProps p = {};
+    p.allocType = cudaMemAllocationTypePinned;
+    p.location.type = cudaMemLocationTypeDevice;
+    p.location.id = device;
+    uint64_t keep = 16ull << 20;
+    if (cudaMemPoolCreate(&pools[device], &p) != cudaSuccess ||
+        cudaMemPoolSetAttribute(pools[device], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaGetLastError();
+      pools[device] = nullptr;
+    }
+  }
+  return pools[device];
+}
+
+void closure_trim(int device) {
+  if (cudaMemPool_t p = work_pool(device, false)) cudaMemPoolTrimTo(p, 0);
+}
+
 struct StreamBuf {
   void* p = nullptr;
   cudaStream_t s;
+  bool pooled = false;
   StreamBuf(size_t bytes, cudaStream_t st) : s(st) {
-    if (cudaMallocAsync(&p, bytes, s) != cudaSuccess) {
-      cudaGetLastError();
-      p = nullptr;
-    }
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaMemPool_t pool = work_pool(dev, true);
+    pooled = pool && cudaMallocFromPoolAsync(&p, bytes, pool, s) == cudaSuccess;
+    if (!pooled && cudaMalloc(&p, bytes) != cudaSuccess) p = nullptr;
+    if (!pooled) cudaGetLastError();
   }
   ~StreamBuf() {
-    if (p) cudaFreeAsync(p, s);
+    if (p && pooled) cudaFreeAsync(p, s);
+    else if (p) cudaFree(p);
   }
   float* f() const { return (float*)p; }
 };
@@ -770,33 +838,18 @@ lbm_status lbm_closure_train(const float* feats, const float* targets, int64_t n
     k_stats<<<SG, 256, 0, s>>>(feats, targets, n, spart);
     k_stats_final<<<MLP_IN + 1, 256, 0, s>>>(feats, targets, n, spart, SG, stats);
     for (int it = 1; it <= steps; ++it) {
-      k_minibatch<<<G, 256, 0, s>>>(theta_io, feats, targets, n, nullptr, seed, (int64_t)(it - 1) * batch,
-                                    batch, stats, part);
+      launch_step(it > 1, k_minibatch, G, 256, 0, s, theta_io, feats, targets, n, nullptr, seed,
+                  (int64_t)(it - 1) * batch, batch, stats, part);
       const float c1 = 1.f - powf(0.9f, (float)it), c2 = 1.f - powf(0.999f, (float)it);
-      k_reduce<true><<<REDUCE_CTAS, 256, 0, s>>>(part, G, batch, nullptr, theta_io, m, v, lr, c1, c2, loss);
+      launch_step(true, k_reduce<true>, REDUCE_CTAS, 256, 0, s, part, G, batch, nullptr, theta_io, m, v, lr, c1,
+                  c2, loss);
     }
-    if (loss_out) cudaMemcpyAsync(loss_out, loss, sizeof(float), cudaMemcpyDeviceToHost, s);
-    // fold the normalisation into the first and last layers
-    std::vector<float> th(MLP_PARAMS), sv(2 * MLP_IN + 2);
-    cudaMemcpyAsync(th.data(), theta_io, MLP_PARAMS * 4, cudaMemcpyDeviceToHost, s);
-    cudaMemcpyAsync(sv.data(), stats, sv.size() * 4, cudaMemcpyDeviceToHost, s);
-    cudaError_t e = cudaStreamSynchronize(s);
+    k_fold<<<1, MLP_H, 0, s>>>(theta_io, stats);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && loss_out)
+      e = cudaMemcpyAsync(loss_out, loss, sizeof(float), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) st = cuda_fail(e, "closure_train");
-    if (!st) {
-      for (int j = 0; j < MLP_H; ++j) {
-        double b = th[P_B1 + j];
-        for (int k = 0; k < MLP_IN; ++k) {
-          b -= (double)th[P_W1 + j * MLP_IN + k] * sv[k] / sv[MLP_IN + k];
-          th[P_W1 + j * MLP_IN + k] /= sv[MLP_IN + k];
-        }
-        th[P_B1 + j] = (float)b;
-        th[P_W3 + j] *= sv[2 * MLP_IN + 1];
-      }
-      th[P_B3] = th[P_B3] * sv[2 * MLP_IN + 1] + sv[2 * MLP_IN];
-      e = cudaMemcpyAsync(theta_io, th.data(), MLP_PARAMS * 4, cudaMemcpyHostToDevice, s);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-      if (e != cudaSuccess) st = cuda_fail(e, "closure_train fold");
-    }
   }
   return st;
 }
