@@ -325,8 +325,11 @@ static lbm_status dense_step_t(Grid& g, Level& L, cudaStream_t s) {
     // kernel on the grid's high-priority group stream: both read the
     // previous state and write disjoint voxels
     // (one launch holds both groups for the scalar kernel, unless their times
-    // are recorded)
+    // are recorded; with 16-bit storage only on small grids, as the boundary
+    // code costs the interior's 48 registers a spill: 256^3 FP16 cavity 266 ->
+    // 292 us a step, while a second stream costs 3 us)
     const bool one = !vec_ok && !g.prof && L.n_reg > 0 && zc > 0 && L.nz < 65535 &&
+                     (S == S_F32 || L.n_slots <= (1 << 21)) &&
                      (int64_t)gx * gy * 256 * (65535 - zc) >= L.n_reg;
     const bool fork = L.n_reg > 0 && zc > 0 && !one;
     cudaStream_t sb = s;
