@@ -419,13 +419,15 @@ __device__ __forceinline__ void sparse_update(const SparseArgs& a, int64_t slot)
 // BOUNDARY_BM with 8^3 blocks takes one block per CTA (two voxels per
 // thread): the launch over every block, most of which leave at once on
 // their boundary bit, then has half as many CTAs.
-// Resident CTAs per SM of the lean kernels: the 16-bit, 32-bit-offset D3Q19
-// form fits in 40 registers without spilling and runs 6 (measured +6 % on
-// the FP16 sphere channel against 5); with 64-bit offsets it stays at 5.
+// Resident CTAs per SM of the lean kernels, which are bound by latency as long
+// as the registers hold: D3Q19 fits in 40 without spilling and runs 6 (512 x 256
+// x 256 channel, FP32: 4 CTAs 294, 5 273, 6 265, 7 with a spill 277 us a step;
+// 16-bit with 64-bit offsets stays at 5), D3Q27 in 64 and runs 4 (half-size
+// FP32 REG channel: 3 CTAs 70.5, 4 63.4, 5 with a spill 72.8).
 template <int S, int MODE, class IDX>
 constexpr int sparse_min_ctas() {
   return (MODE == MODE_INTERIOR || MODE == MODE_INTERIOR_BM)
-             ? (Q == 27 ? 3 : (S == S_F32 ? 4 : (MODE == MODE_INTERIOR && sizeof(IDX) == 4 ? 6 : 5)))
+             ? (Q == 27 ? 4 : (S == S_F32 ? 6 : (MODE == MODE_INTERIOR && sizeof(IDX) == 4 ? 6 : 5)))
              : 1;
 }
 
@@ -503,8 +505,12 @@ template <> struct Pair16<S_BF16> {
   __device__ static __forceinline__ T2 pack(float a, float b) { return __floats2bfloat162_rn(a, b); }
 };
 
+//
+// Five CTAs per SM: with 48 registers BGK spills 48 bytes, and still the FP16
+// channel takes 174 us a step against 178 at four (REG, no spill: 173 against
+// 184); six spill 212 bytes and take 232.
 template <int S, int COLL, bool GROUP>
-__global__ void __launch_bounds__(SP_THREADS, 4) sparse_pair16(SparseArgs a) {
+__global__ void __launch_bounds__(SP_THREADS, 5) sparse_pair16(SparseArgs a) {
   static_assert(Q == 19 && S != S_F32, "two-voxel kernel: D3Q19, 16-bit storage");
   using T = typename Codec<S>::T;
   using P = Pair16<S>;
