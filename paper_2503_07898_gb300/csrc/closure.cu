@@ -478,9 +478,9 @@ struct DevBuf {
   float* f() const { return (float*)p; }
 };
 
-// A training call's workspace, from a stream-ordered pool per device that keeps at
-// most 16 MB between calls (a call needs up to 7 MB; mapping them anew cost
-// 150 us of it) and gives them back when a grid is destroyed.
+// A training call's workspace (up to 7 MB), from a stream-ordered pool per device
+// that keeps at most 64 MB between calls (pools grow by 32 MB; mapping them anew
+// took 200 us of every call) and gives them back when a grid is destroyed.
 static cudaMemPool_t work_pool(int device, bool create) {
   static std::mutex m;
   static cudaMemPool_t pools[64] = {};
@@ -491,7 +491,7 @@ static cudaMemPool_t work_pool(int device, bool create) {
     p.allocType = cudaMemAllocationTypePinned;
     p.location.type = cudaMemLocationTypeDevice;
     p.location.id = device;
-    uint64_t keep = 16ull << 20;
+    uint64_t keep = 64ull << 20;
     if (cudaMemPoolCreate(&pools[device], &p) != cudaSuccess ||
         cudaMemPoolSetAttribute(pools[device], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
       cudaGetLastError();
