@@ -91,7 +91,8 @@ __global__ void __launch_bounds__(256, S == S_F32 ? 4 : 5) dense_interior(DenseA
   // D3Q27)
   if (lean_row(a, y, z)) {
     if constexpr (S == S_F32) {
-      if (wm) pull_row_interior<S, IDX, true>((const T*)a.fin, a, x, y, z, (IDX)v, wm, g);
+      // one form per warp: a lane without wall bits selects nothing
+      if (__any_sync(__activemask(), wm != 0u)) pull_row_interior<S, IDX, true>((const T*)a.fin, a, x, y, z, (IDX)v, wm, g);
       else pull_row_interior<S, IDX, false>((const T*)a.fin, a, x, y, z, (IDX)v, 0u, g);
     } else {
       pull_lean<S, IDX>(a, x, y, z, (IDX)v, wm, g, [&](auto ic, IDX o) {

@@ -129,34 +129,33 @@ __device__ __forceinline__ void pull_lean(const DenseArgs& a, int x, int y, int 
     else if constexpr (cz(I) < 0) o += zn;
     return o;
   };
-  static_for<Q>([&](auto ic) {
-    constexpr int I = decltype(ic)::value;
-    g[I] = Codec<S>::template load<I>(at(ic, src(ic)));
-  });
+  // raw values first, so that a re-read waits for nothing but its own loads
+  typename Codec<S>::T r[Q];
+  static_for<Q>([&](auto ic) { r[decltype(ic)::value] = at(ic, src(ic)); });
   if (x == 0) {  // c_x = +1: the source lies past the row start
     static_for<Q>([&](auto ic) {
       constexpr int I = decltype(ic)::value;
-      if constexpr (cx(I) > 0)
-        g[I] = Codec<S>::template load<I>(a.px ? at(ic, src(ic) + nx)
-                                               : at(IC<opp(I)>{}, v - (IDX)cx(I)));
+      if constexpr (cx(I) > 0) r[I] = a.px ? at(ic, src(ic) + nx) : at(IC<opp(I)>{}, v - (IDX)cx(I));
     });
   }
   if (x == a.nx - 1) {  // c_x = -1: the source lies past the row end
     static_for<Q>([&](auto ic) {
       constexpr int I = decltype(ic)::value;
-      if constexpr (cx(I) < 0)
-        g[I] = Codec<S>::template load<I>(a.px ? at(ic, src(ic) - nx)
-                                               : at(IC<opp(I)>{}, v - (IDX)cx(I)));
+      if constexpr (cx(I) < 0) r[I] = a.px ? at(ic, src(ic) - nx) : at(IC<opp(I)>{}, v - (IDX)cx(I));
     });
   }
   if (wm) {  // sources on walls: halfway bounce-back
     static_for<Q>([&](auto ic) {
       constexpr int I = decltype(ic)::value;
       if constexpr (I != 0) {
-        if ((wm >> I) & 1u) g[I] = Codec<S>::template load<I>(at(IC<opp(I)>{}, v - (IDX)cx(I)));
+        if ((wm >> I) & 1u) r[I] = at(IC<opp(I)>{}, v - (IDX)cx(I));
       }
     });
   }
+  static_for<Q>([&](auto ic) {
+    constexpr int I = decltype(ic)::value;
+    g[I] = Codec<S>::template load<I>(r[I]);
+  });
 }
 
 // A row of the lean pull: no non-periodic box side next to it in y or z.
