@@ -106,9 +106,9 @@ __device__ __forceinline__ void load_raw(const typename Codec<S>::T* in, int64_t
 // that pipe (29 us per operation and voxel at 256^3: some 190, 125 and 68 of
 // them); with the exact sums and pairs of floats they move DRAM traffic.
 // Measured on GB300, 256^3 FP32, init + moments + conservation: 10.49 ms ->
-// 1.09 ms (DRAM floor 0.73 ms).
+// 1.04 ms (DRAM floor 0.73 ms).
 template <int S, bool DENSE>
-__global__ void __launch_bounds__(256) k_init_eq(LevelDev d, void* f, const double* __restrict__ rho,
+__global__ void __launch_bounds__(256, 6) k_init_eq(LevelDev d, void* f, const double* __restrict__ rho,
                                                  const double* __restrict__ u) {
   using T = typename Codec<S>::T;
   const int64_t n = (int64_t)d.nx * d.ny * d.nz;
@@ -189,12 +189,15 @@ __global__ void k_decode(LevelDev d, const void* f, double* dst) {
 // Pass 1: every CTA reduces a fixed, grid-strided set of slots to 4 doubles
 // (per thread an exact 64-bit fixed-point sum and, for voxels outside its
 // window, an FP64 one; then warp shuffles and shared memory) and writes them
-// to partials[cta].  A thread adds at most N / 311,296 voxels below 2^46
+// to partials[cta].  A thread adds at most N / 233,472 voxels below 2^46
 // units each: no overflow.
 // Pass 2: one CTA adds the partials in a fixed order.  The result does not
 // depend on scheduling, so repeated calls give bit-identical sums.
 constexpr int RED_THREADS = 256;
-constexpr int RED_CTAS = kRedCtas;
+// Six CTAs per SM, all resident: 258 us at 256^3 FP32 (307 with 1216 CTAs, four
+// resident per SM).
+constexpr int RED_CTAS = 912;
+static_assert(RED_CTAS <= kRedCtas, "partials of one level");
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -203,7 +206,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 template <int S>
-__global__ void __launch_bounds__(RED_THREADS) k_cons_partial(LevelDev d, const void* f,
+__global__ void __launch_bounds__(RED_THREADS, 6) k_cons_partial(LevelDev d, const void* f,
                                                               double weight, double* partials) {
   using T = typename Codec<S>::T;
   const T* in = (const T*)f;
