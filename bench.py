@@ -687,6 +687,11 @@ def run_ours(args, rank, world, local_rank):
     stats = lbm.lbm_profile_read(g)
     lbm.lbm_profile(g, 0)
     launches_per_step = sum(s["launches"] for s in stats.values()) / kb
+    # only profiled steps give each group its own launch: the scalar kernel holds
+    # both in one with FP32 storage, and with 16-bit storage up to 2^21 voxels
+    if (args.schedule == "disaggregated" and lbm.VARIANT_NAMES[variant] == "scalar"
+            and (args.storage == "f32" or n ** 3 <= 1 << 21)):
+        launches_per_step = 1
     top = max(stats, key=lambda k: stats[k]["total_ms"])
     st = stats[top]
     bpu = BYTES_PER_UPDATE[args.storage]
