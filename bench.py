@@ -44,8 +44,8 @@ METRIC = "D3Q19 GLUPS & % HBM roofline, FP32 vs FP16-store/learned at stated err
 # only while the kernel sources hash to the recorded value: the 160^3
 # capture of dense_interior (dram__bytes_read.sum + dram__bytes_write.sum,
 # 4,070,400 updates per launch) scaled by units to one 256^3 launch
-# (16,711,680 updates), profiles/dense_interior_cavity160_ncu.md; keyed by
-# kernel and storage (the FP16 capture: dense_interior_f16_cavity160_ncu.md).
+# (16,711,680 updates), profiles/f16_kernels_current_ncu.md (FP32 from the launch
+# that holds both groups, 4,096,000 updates); keyed by kernel and storage.
 NCU_TRAFFIC = {("dense_interior", "f32"): {"bytes_per_launch": 2.345015e+09, "src_sha": "ef0bcf0720e1da82"},
                ("dense_interior", "f16"): {"bytes_per_launch": 1.109753e+09, "src_sha": "ef0bcf0720e1da82"}}
 
