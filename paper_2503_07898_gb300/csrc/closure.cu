@@ -540,23 +540,55 @@ struct DsArgs {
 // 230 operations per fine voxel and 350 per coarse one at two per SM and
 // clock); as exact sums and pairs of floats (exact.cuh; results rounded to
 // FP32, as before) they cost FP32 operations only.  Measured on GB300, 256^3
-// FP32, r = 2, dataset + statistics + 20 training steps: 11.2 ms -> 1.4 ms.
+// FP32, r = 2, one dataset call: 8.5 ms -> 0.55 ms.
 
-// rho and j of a fine voxel outside the exact sums' window, from FP64.
-__device__ __noinline__ void filter_wide(const float v[Q], bool shifted, DD* out) {
-  double m = 0, x = 0, y = 0, z = 0;
-  for (int i = 0; i < Q; ++i) {
-    const double f = shifted ? wd(i) + (double)v[i] : (double)v[i];
-    m += f;
-    x += cx(i) * f;
-    y += cy(i) * f;
-    z += cz(i) * f;
-  }
-  const double d[4] = {m, x, y, z};
-  for (int k = 0; k < 4; ++k) {
-    out[k].h = (float)d[k];
-    out[k].l = (float)(d[k] - (double)out[k].h);
-  }
+// Coordinates of the calling thread's coarse voxel; false past the end.
+__device__ __forceinline__ bool cvoxel(const DsArgs& a, int64_t& X, int& x, int& y, int& z) {
+  X = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (X >= (int64_t)a.cx_ * a.cy_ * a.cz_) return false;
+  const int row = (int)(X / a.cx_);
+  x = (int)(X - (int64_t)row * a.cx_);
+  z = row / a.cy_;
+  y = row - z * a.cy_;
+  return true;
+}
+
+// One coarse voxel's filter in FP64.
+template <int S> __device__ __noinline__ void filter_f64(const DsArgs& a, int64_t X, int Xx, int Xy, int Xz) {
+  using T = typename Codec<S>::T;
+  const int64_t nc = (int64_t)a.cx_ * a.cy_ * a.cz_;
+  double sp[Q], m[10];
+  for (int i = 0; i < Q; ++i) sp[i] = 0;
+  for (int k = 0; k < 10; ++k) m[k] = 0;
+  for (int dz = 0; dz < a.r; ++dz)
+    for (int dy = 0; dy < a.r; ++dy) {
+      const T* f = (const T*)a.f + (Xx * a.r + (int64_t)a.nx * ((Xy * a.r + dy) + (int64_t)a.ny * (Xz * a.r + dz)));
+      for (int dx = 0; dx < a.r; ++dx, ++f) {
+        double rho = 0, jx = 0, jy = 0, jz = 0;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+          const double fi = Codec<S>::abs_d(f[(int64_t)i * a.N], i);
+          sp[i] += fi - wd(i);
+          rho += fi;
+          jx += cx(i) * fi;
+          jy += cy(i) * fi;
+          jz += cz(i) * fi;
+        }
+        m[0] += rho;
+        m[1] += jx;
+        m[2] += jy;
+        m[3] += jz;
+        m[4] += jx * jx / rho;
+        m[5] += jy * jy / rho;
+        m[6] += jz * jz / rho;
+        m[7] += jx * jy / rho;
+        m[8] += jx * jz / rho;
+        m[9] += jy * jz / rho;
+      }
+    }
+  const double inv = 1.0 / ((double)a.r * a.r * a.r);
+  for (int i = 0; i < Q; ++i) a.sbar[(int64_t)i * nc + X] = (float)(sp[i] * inv);
+  for (int k = 0; k < 10; ++k) a.mom[(int64_t)k * nc + X] = (float)(m[k] * inv);
 }
 
 // mean of n values whose sum is s, minus w, to FP32.  pow2: n is a power of two
@@ -572,22 +604,55 @@ __device__ __forceinline__ float mean_minus(DD s, float n, bool pow2, DD inv_n, 
   return dd_mul(t, inv_n).h;
 }
 
-// One thread per coarse voxel.  rho and j of each fine voxel are exact.  The
-// population sums add the split parts: up to 8^3 upper parts stay below 2^24
-// units and the lower ones round at 2^-34 at worst.  LARGE (r > 8): they
-// collect every rounding error instead (dd_acc).
-template <int S, bool LARGE>
-__global__ void __launch_bounds__(128) k_ds_filter(DsArgs a) {
+// rho and j of a fine voxel outside the exact sums' window, from FP64.  False if
+// pairs of floats cannot go on with them (infinities, NaN, magnitudes that
+// products or quotients would carry out of FP32's range).
+__device__ __noinline__ bool filter_wide(const float v[Q], bool shifted, DD* out) {
+  double m = 0, x = 0, y = 0, z = 0;
+  bool in = true;
+  for (int i = 0; i < Q; ++i) {
+    in = in && fabsf(v[i]) < 0x1p30f;
+    const double f = shifted ? wd(i) + (double)v[i] : (double)v[i];
+    m += f;
+    x += cx(i) * f;
+    y += cy(i) * f;
+    z += cz(i) * f;
+  }
+  const double d[4] = {m, x, y, z};
+  for (int k = 0; k < 4; ++k) {
+    out[k].h = (float)d[k];
+    out[k].l = (float)(d[k] - (double)out[k].h);
+  }
+  return in && fabs(m) > 0x1p-30;
+}
+
+// One thread per coarse voxel.  rho and j of each fine voxel are exact.  The sums
+// over the fine voxels:
+//   r <= 3, FP32 and FP16: the population sums add the split parts without
+//     rounding (per voxel an upper part counts at most 2^15 (FP32) or 2^19 (FP16)
+//     units, a lower one 2^19, and 2^19 r^3 <= 2^24).  A coarse voxel with a
+//     value outside the window takes the FP64 form as a whole;
+//   PAIRS, r <= 16: pairs of floats, renormalised after each row, so that their
+//     error stays below r^4 2^-48 of the sum of magnitudes (2^-32); any
+//     magnitude will do, and voxels outside the window take rho and j from
+//     FP64.  BF16 takes this form at r <= 3 too: its values reach below the
+//     window wherever s crosses zero.
+// Wider filters are left to the FP64 form.  One dataset call at 256^3, r = 2,
+// FP32 and FP16: 0.55 ms with the split parts, 0.67 with pairs; r = 4: 0.45
+// (FP64: 6.9 and 7.5).
+template <int S, bool PAIRS>
+__global__ void __launch_bounds__(128) k_ds_filter(const __grid_constant__ DsArgs a) {
   using T = typename Codec<S>::T;
   const int64_t nc = (int64_t)a.cx_ * a.cy_ * a.cz_;
-  const int64_t X = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (X >= nc) return;
-  const int row = (int)(X / a.cx_), Xx = (int)(X - (int64_t)row * a.cx_), Xz = row / a.cy_, Xy = row - Xz * a.cy_;
+  int64_t X;
+  int Xx, Xy, Xz;
+  if (!cvoxel(a, X, Xx, Xy, Xz)) return;
   DD sp[Q], m[10];
 #pragma unroll
   for (int i = 0; i < Q; ++i) sp[i] = {0.f, 0.f};
 #pragma unroll
   for (int k = 0; k < 10; ++k) m[k] = {0.f, 0.f};
+  bool in = true;
 #pragma unroll 1
   for (int dz = 0; dz < a.r; ++dz)
 #pragma unroll 1
@@ -606,10 +671,10 @@ __global__ void __launch_bounds__(128) k_ds_filter(DsArgs a) {
         {
           float h[Q], l[Q];
           const bool ok = FixSum<S>::split(v, h, l);
-          if (!q.pairs(h, l, ok, c)) filter_wide(v, S != S_F32, c);
+          if (!q.pairs(h, l, ok, c)) in = PAIRS && filter_wide(v, S != S_F32, c) && in;
 #pragma unroll
           for (int i = 0; i < Q; ++i) {
-            if constexpr (LARGE) {
+            if constexpr (PAIRS) {
               dd_acc(sp[i], v[i]);
             } else {
               sp[i].h = add_rn(sp[i].h, h[i]);
@@ -628,8 +693,18 @@ __global__ void __launch_bounds__(128) k_ds_filter(DsArgs a) {
         dd_acc(m[8], dd_prod(c[1], uz));
         dd_acc(m[9], dd_prod(c[2], uz));
       }
+      if constexpr (PAIRS) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) sp[i] = two_sum(sp[i].h, sp[i].l);
+#pragma unroll
+        for (int k = 0; k < 10; ++k) m[k] = two_sum(m[k].h, m[k].l);
+      }
     }
-  const float n = (float)((int64_t)a.r * a.r * a.r);
+  if (!in) {
+    filter_f64<S>(a, X, Xx, Xy, Xz);
+    return;
+  }
+  const float n = (float)(a.r * a.r * a.r);
   const DD inv = dd_inv({n, 0.f});
   const bool pow2 = (a.r & (a.r - 1)) == 0;
   static_for<Q>([&](auto ic) {
@@ -642,25 +717,22 @@ __global__ void __launch_bounds__(128) k_ds_filter(DsArgs a) {
   for (int k = 0; k < 10; ++k) a.mom[(int64_t)k * nc + X] = mean_minus(m[k], n, pow2, inv, 0.f, 0.f);
 }
 
+template <int S> __global__ void __launch_bounds__(128) k_ds_filter_f64(const __grid_constant__ DsArgs a) {
+  int64_t X;
+  int x, y, z;
+  if (cvoxel(a, X, x, y, z)) filter_f64<S>(a, X, x, y, z);
+}
+
 template <int S> static void ds_filter(const DsArgs& a, unsigned nb, cudaStream_t s) {
-  if (a.r > 8) k_ds_filter<S, true><<<nb, 128, 0, s>>>(a);
-  else k_ds_filter<S, false><<<nb, 128, 0, s>>>(a);
+  if (a.r <= 3 && S != S_BF16) k_ds_filter<S, false><<<nb, 128, 0, s>>>(a);
+  else if (a.r <= 16) k_ds_filter<S, true><<<nb, 128, 0, s>>>(a);
+  else k_ds_filter_f64<S><<<nb, 128, 0, s>>>(a);
 }
 
 // Index of a coarse voxel with every coordinate in [-1, c].
 __device__ __forceinline__ int64_t cidx(const DsArgs& a, int x, int y, int z) {
   auto wrap = [](int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); };
   return wrap(x, a.cx_) + (int64_t)a.cx_ * (wrap(y, a.cy_) + (int64_t)a.cy_ * wrap(z, a.cz_));
-}
-// Coordinates of the calling thread's coarse voxel; false past the end.
-__device__ __forceinline__ bool cvoxel(const DsArgs& a, int64_t& X, int& x, int& y, int& z) {
-  X = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (X >= (int64_t)a.cx_ * a.cy_ * a.cz_) return false;
-  const int row = (int)(X / a.cx_);
-  x = (int)(X - (int64_t)row * a.cx_);
-  z = row / a.cy_;
-  y = row - z * a.cy_;
-  return true;
 }
 
 __global__ void __launch_bounds__(128) k_ds_features(DsArgs a, float tau, float* feats) {
