@@ -832,19 +832,17 @@ __global__ void __launch_bounds__(128) k_ds_target(DsArgs a, float tau, float* t
         dd_acc(n, a.num[i]);
         dd_acc(d, a.den[i]);
       }
-  n = quick_sum(n.h, n.l);
+  n = two_sum(n.h, n.l);  // n may cancel
   d = quick_sum(d.h, d.l);
   float t = 0.f;
-  if (d.h > 0.f) {
-    const float lo = (float)(-((double)tau - 0.5) + 1e-3);
-    if (d.h > 1e-30f) {
-      const DD q = dd_mul(n, dd_inv(d)), p = two_prod(-3.f, q.h);
-      t = add_rn(p.h, fmaf(-3.f, q.l, p.l));
-    } else {  // 1 / d would overflow
-      t = (float)(-3.0 * ((double)n.h + n.l) / ((double)d.h + d.l));
-    }
-    t = t < lo ? lo : (t > 0.5f ? 0.5f : t);
+  if (d.h > 1e-30f) {
+    const DD q = dd_mul(n, dd_inv(d)), p = two_prod(-3.f, q.h);
+    t = add_rn(p.h, fmaf(-3.f, q.l, p.l));
+  } else if (d.h > 0.f) {  // 1 / d would overflow
+    t = (float)(-3.0 * ((double)n.h + n.l) / ((double)d.h + d.l));
   }
+  const float lo = (float)(-((double)tau - 0.5) + 1e-3);
+  t = t < lo ? lo : (t > 0.5f ? 0.5f : t);
   targets[X] = t;
 }
 

@@ -78,3 +78,17 @@ def test_infinite_population(lbm, r):
     assert F[hit, 0] == np.inf
     rest = np.arange(len(F)) != hit
     assert np.array_equal(F[rest], clean[rest])
+
+
+@pytest.mark.parametrize("tau", [0.5005, 0.501, 0.75])
+def test_target_bounds_without_gradients(lbm, tau):
+    """No velocity gradient: the target is 0 brought into its bounds, whose lower
+    one is positive for tau < 0.501."""
+    dims = (8, 12, 16)
+    g = lbm.lbm_grid_create_dense(dims, lbm.physics(0.52, periodic=(1, 1, 1)))
+    lbm.lbm_init_equilibrium(g, 0, np.ones(dims[::-1]), np.zeros((3,) + dims[::-1]))
+    f = lbm.lbm_get_populations_f64(g, 0)
+    _, T = dataset(lbm, g, dims, 2, tau)
+    lbm.lbm_grid_destroy(g)
+    want = ocl.eddy_target(f, 2, float(np.float32(tau))).ravel()
+    assert np.array_equal(T, want.astype(np.float32))
