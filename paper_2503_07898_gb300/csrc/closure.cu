@@ -364,16 +364,22 @@ __global__ void __launch_bounds__(256) k_reduce(const float* __restrict__ part, 
 // coalesced) and sums v - k and (v - k)^2 as pairs of floats, k = the column's
 // first value: the variance does not cancel against a large mean, which the
 // FP64 sums of v and v^2 did, on 17 CTAs.  Bound by DRAM (68 bytes per sample).
+// The largest |v - k| goes along: k_stats_final sums a column again in FP64
+// where squares have left FP32's range or k is far out.
 constexpr int STAT_CTAS = 1216;  // eight per SM: the chains of dependent additions need the warps
+constexpr int STAT_SUMS = 3 * (MLP_IN + 1);  // per CTA: sums of v - k and (v - k)^2, largest |v - k|
 __global__ void __launch_bounds__(256) k_stats(const float* __restrict__ X,
                                                const float* __restrict__ T, int64_t n,
                                                double* __restrict__ part) {
   __shared__ double sh[2][16][17];
   __shared__ double st[2][256];
+  __shared__ float mh[16][17], mt[256];
   const int c = threadIdx.x & 15, r = threadIdx.x >> 4;
   DD s1 = {0.f, 0.f}, s2 = {0.f, 0.f}, t1 = {0.f, 0.f}, t2 = {0.f, 0.f};
-  auto take = [](DD& a, DD& b, float v, float k) {
+  float sm = 0.f, tm = 0.f;
+  auto take = [](DD& a, DD& b, float& m, float v, float k) {
     const DD d = two_sum(v, -k);
+    m = fmaxf(m, fabsf(d.h));
     dd_acc(a, d);
     const DD q = two_prod(d.h, d.h);
     dd_acc(b, {q.h, fmaf(2.f * d.h, d.l, q.l)});
@@ -383,15 +389,18 @@ __global__ void __launch_bounds__(256) k_stats(const float* __restrict__ X,
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int64_t i = i0 + 16 * u + r;
-      if (i < n) take(s1, s2, X[i * MLP_IN + c], kx);
+      if (i < n) take(s1, s2, sm, X[i * MLP_IN + c], kx);
     }
-    if (threadIdx.x < 64 && i0 + threadIdx.x < n) take(t1, t2, T[i0 + threadIdx.x], kt);
+    if (threadIdx.x < 64 && i0 + threadIdx.x < n) take(t1, t2, tm, T[i0 + threadIdx.x], kt);
   }
   sh[0][r][c] = (double)s1.h + s1.l;
   sh[1][r][c] = (double)s2.h + s2.l;
   st[0][threadIdx.x] = (double)t1.h + t1.l;
   st[1][threadIdx.x] = (double)t2.h + t2.l;
+  mh[r][c] = sm;
+  mt[threadIdx.x] = tm;
   __syncthreads();
+  double* o = part + (int64_t)blockIdx.x * STAT_SUMS;
   if (threadIdx.x < 34) {
     const int k = threadIdx.x / 17, j = threadIdx.x - 17 * k;
     double a = 0.0;
@@ -399,37 +408,84 @@ __global__ void __launch_bounds__(256) k_stats(const float* __restrict__ X,
       for (int q = 0; q < 16; ++q) a += sh[k][q][j];
     else
       for (int q = 0; q < 64; ++q) a += st[k][q];
-    part[(int64_t)blockIdx.x * 34 + threadIdx.x] = a;
+    o[threadIdx.x] = a;
+  } else if (threadIdx.x >= 64 && threadIdx.x < 64 + 17) {
+    const int j = threadIdx.x - 64;
+    float m = 0.f;
+    if (j < MLP_IN)
+      for (int q = 0; q < 16; ++q) m = fmaxf(m, mh[q][j]);
+    else
+      for (int q = 0; q < 64; ++q) m = fmaxf(m, mt[q]);
+    o[34 + j] = m;
   }
 }
 
-// One CTA per column adds the CTAs' sums in a fixed order.
+// Sums of a and b (and the largest m) over the CTA's 256 threads, in a fixed order,
+// valid in thread 0.
+__device__ __forceinline__ void stat_sums(double& a, double& b, float& m) {
+  __shared__ double sa[8], sb[8];
+  __shared__ float sm[8];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    sa[threadIdx.x >> 5] = a;
+    sb[threadIdx.x >> 5] = b;
+    sm[threadIdx.x >> 5] = m;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int w = 1; w < 8; ++w) {
+      a += sa[w];
+      b += sb[w];
+      m = fmaxf(m, sm[w]);
+    }
+}
+
+// One CTA per column adds the CTAs' sums in a fixed order.  The pairs of floats
+// are good to 2^-41 of each sum.  FP64 takes the column instead
+//  - when a sum is not finite (|v - k| above 2^63, infinities, NaN);
+//  - when the mean square of v - k is below 1e-30, where the low parts of the
+//    squares leave FP32's range (but not for a constant column);
+//  - when k is more than 32 deviations from the mean: b / n - d^2 would cancel
+//    ten bits and more.
 __global__ void __launch_bounds__(256) k_stats_final(const float* X, const float* T, int64_t n,
                                                     const double* __restrict__ part, int G,
                                                     float* stats) {
   const int c = blockIdx.x;  // 0..16 (16 = target)
   double a = 0.0, b = 0.0;
+  float m = 0.f;
   for (int g = threadIdx.x; g < G; g += 256) {
-    a += part[(int64_t)g * 34 + c];
-    b += part[(int64_t)g * 34 + 17 + c];
+    const double* p = part + (int64_t)g * STAT_SUMS + c;
+    a += p[0];
+    b += p[17];
+    m = fmaxf(m, (float)p[34]);
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(0xffffffffu, a, o);
-    b += __shfl_xor_sync(0xffffffffu, b, o);
-  }
-  __shared__ double sa[8], sb[8];
-  if ((threadIdx.x & 31) == 0) {
-    sa[threadIdx.x >> 5] = a;
-    sb[threadIdx.x >> 5] = b;
+  stat_sums(a, b, m);
+  __shared__ double mid;
+  __shared__ bool again;
+  double k = (double)(c < MLP_IN ? X[c] : T[0]);
+  if (threadIdx.x == 0) {
+    const double d = a / (double)n, ms = b / (double)n;
+    again = !(isfinite(a) && isfinite(b)) || (m > 0.f && ms < 1e-30) || d * d > 1024.0 * (ms - d * d);
+    mid = isfinite(k + d) ? k + d : 0.0;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) {
-      a += sa[w];
-      b += sb[w];
+  if (again) {
+    k = mid;
+    a = b = 0.0;
+    for (int64_t i = threadIdx.x; i < n; i += 256) {
+      const double v = (double)(c < MLP_IN ? X[i * MLP_IN + c] : T[i]) - k;
+      a += v;
+      b += v * v;
     }
-    const double d = a / (double)n, mean = (double)(c < MLP_IN ? X[c] : T[0]) + d;
+    stat_sums(a, b, m);
+  }
+  if (threadIdx.x == 0) {
+    const double d = a / (double)n, mean = k + d;
     double var = b / (double)n - d * d;
     double sd = var > 0 ? sqrt(var) : 0.0;
     // constant column (the tau feature of a one-level set): a deviation below
@@ -905,7 +961,7 @@ lbm_status lbm_closure_train(const float* feats, const float* targets, int64_t n
   // and the column statistics
   const int G = minibatch_ctas(batch);
   const size_t n_part = (size_t)G * PART;
-  StreamBuf buf((n_part + 2 * PART + 64) * sizeof(float) + STAT_CTAS * 34 * sizeof(double), s);
+  StreamBuf buf((n_part + 2 * PART + 64) * sizeof(float) + STAT_CTAS * STAT_SUMS * sizeof(double), s);
   lbm_status st = buf.p ? LBM_OK : fail(LBM_ERR_OOM, "device allocation failed");
   if (!st) {
     float *part = buf.f(), *m = part + n_part, *v = m + PART, *stats = v + PART, *loss = stats + 48;
