@@ -182,7 +182,7 @@ template <int S> struct FixSum {
     const bool ok = split(v, h, l);
     sums(h, a);
     sums(l, b);
-    rho = S == S_F32 ? a[0] + b[0] : 1.f + a[0];
+    rho = total(a[0], b[0]);
     return ok && rho >= 0.0625f && rho < 64.f;
   }
   // The two parts of each value (v = h + l always); whether all are in the window.
@@ -215,7 +215,7 @@ template <int S> struct FixSum {
     float a[4], b[4];
     sums(h, a);
     sums(l, b);
-    rho = S == S_F32 ? a[0] + b[0] : 1.f + a[0];
+    rho = total(a[0], b[0]);
     c[0] = two_sum(a[0], b[0]);
     if (S != S_F32) {
       const DD s = two_sum(1.f, c[0].h);
@@ -227,6 +227,10 @@ template <int S> struct FixSum {
   }
 
  private:
+  // rho to FP32 (1 + a is exact): the reciprocal's third-order step needs all 24 bits
+  __host__ __device__ static __forceinline__ float total(float a, float b) {
+    return S == S_F32 ? add_rn(a, b) : add_rn(add_rn(1.f, a), b);
+  }
   __host__ __device__ static __forceinline__ void sums(const float p[Q], float r[4]) {
     float m = p[0], x = 0.f, y = 0.f, z = 0.f;
 #pragma unroll
@@ -255,29 +259,48 @@ template <int S> struct FixSum {
   }
 };
 
+// x / m rounded to nearest, from a double q within two units in its last place:
+// the remainder |x| 2^-e - Q m of q = Q 2^e is a small integer, so 64-bit products
+// and shifts modulo 2^64 give it exactly, and the remainder over m says by how many
+// units q is off.  |x|, m < 2^47, q < 2^52 (no ties: a quotient of such numbers has
+// no 54-bit form).  Next to a power of two, where the unit changes, the quotient
+// is formed anew.  (A correction by two FP64 operations per quotient would cost
+// 170 us at 256^3; the integer one costs 7 to 30.)
+__host__ __device__ __forceinline__ double round_quotient(int64_t x, int64_t m, double q) {
+  constexpr uint64_t FRACTION = ((uint64_t)1 << 52) - 1;
+  const uint64_t b = d_bits(q), low = b & FRACTION;
+  const int shift = 1075 - (int)((b >> 52) & 0x7ffu);  // -e
+  const uint64_t a = (uint64_t)(x < 0 ? -x : x);
+  const int64_t r = (int64_t)((shift < 64 ? a << shift : 0) - (low + FRACTION + 1) * (uint64_t)m);
+  if (x == 0 || r == 0) return q;
+  if (((low + 2) & FRACTION) < 4) return (double)x / (double)m;
+  const int64_t r2 = 2 * r, m3 = 3 * m;
+  return bits_d(b + (uint64_t)((r2 > m) + (r2 > m3) - (r2 < -m) - (r2 < -m3)));
+}
+
 // rho and u = j / rho as doubles: rho is exact; 1 / rho comes from the FP32
-// reciprocal by one third-order step (relative error below 2^-52), u is one
-// product.  Ten FP64 operations; scalings by powers of two and the
-// conversion of the FP32 value go through the exponent bits.
-#ifdef __CUDACC__
+// reciprocal by one third-order step (relative error below 2^-52.9), u is one
+// product, then rounded to nearest.  Ten FP64 operations; scalings by powers of two
+// and the conversion of the FP32 value go through the exponent bits.
 template <int S>
-__device__ __forceinline__ void fix_moments(const FixSum<S>& f, double& r, double& ux, double& uy,
-                                            double& uz) {
+__host__ __device__ __forceinline__ void fix_moments(const FixSum<S>& f, double& r, double& ux, double& uy,
+                                                     double& uz) {
   // |sums| < 2^47: exact as the low mantissa bits of 1.5 2^52
-  auto dbl = [](int64_t v) {
-    return __longlong_as_double(0x4338000000000000LL + v) - 6755399441055744.0;
-  };
+  auto dbl = [](int64_t v) { return bits_d((uint64_t)(0x4338000000000000LL + v)) - 6755399441055744.0; };
   const double m = dbl(f.m);  // rho 2^FRAC, positive
-  r = __hiloint2double(__double2hiint(m) - (FixSum<S>::FRAC << 20), __double2loint(m));
-  const uint32_t b = __float_as_uint(__frcp_rn(f.rho));  // in (1/64, 16]: normal
-  double y = __hiloint2double((int)(b >> 3) + ((896 - FixSum<S>::FRAC) << 20), (int)(b << 29));
+  r = bits_d(d_bits(m) - ((uint64_t)FixSum<S>::FRAC << 52));
+#ifdef __CUDA_ARCH__
+  const uint32_t b = f_bits(__frcp_rn(f.rho));  // in (1/64, 16]: normal
+#else
+  const uint32_t b = f_bits(1.f / f.rho);
+#endif
+  double y = bits_d(((uint64_t)((b >> 3) + (uint32_t)((896 - FixSum<S>::FRAC) << 20)) << 32) | (uint64_t)(b << 29));
   const double e = fma(-m, y, 1.0);
   y = fma(y, fma(e, e, e), y);
-  ux = dbl(f.x) * y;
-  uy = dbl(f.y) * y;
-  uz = dbl(f.z) * y;
+  ux = round_quotient(f.x, f.m, dbl(f.x) * y);
+  uy = round_quotient(f.y, f.m, dbl(f.y) * y);
+  uz = round_quotient(f.z, f.m, dbl(f.z) * y);
 }
-#endif
 
 // ------------------------------------------------------------- equilibrium
 // f^eq_i from double inputs in pairs of floats, before the last rounding: the

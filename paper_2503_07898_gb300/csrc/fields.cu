@@ -106,7 +106,7 @@ __device__ __forceinline__ void load_raw(const typename Codec<S>::T* in, int64_t
 // that pipe (29 us per operation and voxel at 256^3: some 190, 125 and 68 of
 // them); with the exact sums and pairs of floats they move DRAM traffic.
 // Measured on GB300, 256^3 FP32, init + moments + conservation: 10.49 ms ->
-// 1.04 ms (DRAM floor 0.73 ms).
+// 1.05 ms (DRAM floor 0.73 ms).
 template <int S, bool DENSE>
 __global__ void __launch_bounds__(256, 6) k_init_eq(LevelDev d, void* f, const double* __restrict__ rho,
                                                  const double* __restrict__ u) {
@@ -132,9 +132,12 @@ __global__ void __launch_bounds__(256, 6) k_init_eq(LevelDev d, void* f, const d
   }
 }
 
+// Six CTAs per SM (40 registers) against the five that 48 allow: 256^3, D3Q19
+// FP32 402 -> 369 us, FP16 380 -> 369, D3Q27 FP32 495 -> 429, but D3Q27 FP16
+// 412 -> 443, which keeps five.
 template <int S, bool DENSE>
-__global__ void __launch_bounds__(256) k_moments(LevelDev d, const void* f, double* __restrict__ rho,
-                                                 double* __restrict__ u) {
+__global__ void __launch_bounds__(256, Q == 27 && S != S_F32 ? 5 : 6)
+    k_moments(LevelDev d, const void* f, double* __restrict__ rho, double* __restrict__ u) {
   using T = typename Codec<S>::T;
   const int64_t n = (int64_t)d.nx * d.ny * d.nz;
   const double nan = __longlong_as_double(0x7ff8000000000000LL);
