@@ -326,11 +326,14 @@ static lbm_status dense_step_t(Grid& g, Level& L, cudaStream_t s) {
     // kernel on the grid's high-priority group stream: both read the
     // previous state and write disjoint voxels
     // (one launch holds both groups for the scalar kernel, unless their times
-    // are recorded; with 16-bit storage only on small grids, as the boundary
-    // code costs the interior's 48 registers a spill: 256^3 FP16 cavity 266 ->
-    // 292 us a step, while a second stream costs 3 us)
+    // are recorded; where the boundary code makes the interior spill, only on
+    // grids where that costs less than the 3 us of a second stream.  16-bit
+    // storage, 48 registers: up to 2 M voxels (256^3 FP16 cavity 266 -> 292 us a
+    // step; D3Q27 at 80^3 20.0 -> 17.3, 128^3 58.8 -> 57.9).  D3Q27 FP32, 64: up
+    // to 64^3 (12.5 -> 10.8 us; at 112^3 52.8 -> 56.1, at 256^3 535 -> 583))
+    constexpr int64_t one_max = S != S_F32 ? (1 << 21) : (Q == 27 ? (1 << 18) : INT64_MAX);
     const bool one = !vec_ok && !g.prof && L.n_reg > 0 && zc > 0 && L.nz < 65535 &&
-                     (S == S_F32 || L.n_slots <= (1 << 21)) &&
+                     L.n_slots <= one_max &&
                      (int64_t)gx * gy * 256 * (65535 - zc) >= L.n_reg;
     const bool fork = L.n_reg > 0 && zc > 0 && !one;
     cudaStream_t sb = s;
