@@ -419,16 +419,27 @@ __device__ __forceinline__ void sparse_update(const SparseArgs& a, int64_t slot)
 // BOUNDARY_BM with 8^3 blocks takes one block per CTA (two voxels per
 // thread): the launch over every block, most of which leave at once on
 // their boundary bit, then has half as many CTAs.
-// Resident CTAs per SM of the lean kernels, which are bound by latency as long
-// as the registers hold: D3Q19 fits in 40 without spilling and runs 6 (512 x 256
-// x 256 channel, FP32: 4 CTAs 294, 5 273, 6 265, 7 with a spill 277 us a step;
-// 16-bit with 64-bit offsets stays at 5), D3Q27 in 64 and runs 4 (half-size
-// FP32 REG channel: 3 CTAs 70.5, 4 63.4, 5 with a spill 72.8).
-template <int S, int MODE, class IDX>
+// Resident CTAs per SM of the lean kernels, which are bound by latency until the
+// registers run out.  us a step; "big" is a full box just above 2^31 population
+// elements, where offsets take 64 bits:
+//   D3Q19 FP32, 32-bit offsets (512 x 256 x 256 channel): 4 CTAs 294, 5 273,
+//     6 265 (40 registers; no spill, with the boundary group 68-84 bytes on its
+//     path), 7 277
+//   D3Q19 FP32, 64-bit offsets (496 x 496 x 480): 4 CTAs BGK 3038, REG 3099;
+//     6 spill 190-210 bytes with the boundary group: 3277, 3164
+//   D3Q19 16-bit: 6 with 32-bit offsets, 5 with 64-bit ones
+//   D3Q19 FP32, bitmask grouping (always 64-bit offsets, 40-64 bytes): 6 CTAs
+//     317, 4 321
+//   D3Q27 (half-size FP32 REG channel): 3 CTAs 70.5, 4 63.4, 5 with a spill 72.8;
+//     FP32 with 64-bit offsets (440 x 440 x 416, 60-72 bytes at 4): BGK 3 CTAs
+//     3055, 4 3081; REG 3 3104, 4 2980
+template <int S, int COLL, int MODE, class IDX>
 constexpr int sparse_min_ctas() {
-  return (MODE == MODE_INTERIOR || MODE == MODE_INTERIOR_BM)
-             ? (Q == 27 ? 4 : (S == S_F32 ? 6 : (MODE == MODE_INTERIOR && sizeof(IDX) == 4 ? 6 : 5)))
-             : 1;
+  constexpr bool lean = MODE == MODE_INTERIOR, big = lean && sizeof(IDX) == 8;
+  if (!lean && MODE != MODE_INTERIOR_BM) return 1;
+  if (Q == 27) return S == S_F32 && big && COLL == C_BGK ? 3 : 4;
+  if (S == S_F32) return big ? 4 : 6;
+  return lean && !big ? 6 : 5;
 }
 
 // GROUP: the first CTAs of an interior launch update the boundary group (the
@@ -437,7 +448,7 @@ constexpr int sparse_min_ctas() {
 // its two events per step, and a chain of launches overlaps each launch with
 // the one before it (110 x 80 x 80 FP32 sphere channel: 12.5 -> 9.8 us a step).
 template <int S, int E, int COLL, int MODE, class IDX = int64_t, bool GROUP = false>
-__global__ void __launch_bounds__(SP_THREADS, sparse_min_ctas<S, MODE, IDX>())
+__global__ void __launch_bounds__(SP_THREADS, sparse_min_ctas<S, COLL, MODE, IDX>())
     sparse_kernel(SparseArgs a) {
   constexpr int E3 = E * E * E;
   chain();
