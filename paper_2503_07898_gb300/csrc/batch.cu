@@ -48,9 +48,12 @@ constexpr int VPI = BT * VPT; // voxels per work item: 512 (dense: consecutive i
 
 // Registers are bounded so that the default grid (four CTAs per SM) is resident
 // with FP32 storage as well: unbounded it took 110 and ran two (16 cases,
-// FP32: 468 us a step, 343 at 64 registers).
-template <int S, int COLL, bool CLOSURE>
-__global__ void __launch_bounds__(BT, CLOSURE ? 1 : (S == S_F32 ? 4 : 5)) batch_step_kernel(const BatchCase* __restrict__ cases,
+// FP32: 468 us a step, 343 at 64 registers).  FEW (FP32): unbounded, for batches of
+// at most two items per SM, which are resident either way and gain from more loads
+// in flight (BGK dense, one grid: 288 items 5.80 -> 4.67 us a step, 64 items 4.20 ->
+// 3.97; 320 items 5.90 -> 6.93).
+template <int S, int COLL, bool CLOSURE, bool FEW>
+__global__ void __launch_bounds__(BT, CLOSURE || FEW ? 1 : (S == S_F32 ? 4 : 5)) batch_step_kernel(const BatchCase* __restrict__ cases,
                                                         const int32_t* __restrict__ item_case,
                                                         const int32_t* __restrict__ item_local,
                                                         int64_t n_items, int parity,
@@ -185,12 +188,12 @@ __global__ void __launch_bounds__(BT, CLOSURE ? 1 : (S == S_F32 ? 4 : 5)) batch_
   }
 }
 
-template <int S, int COLL, bool CLOSURE>
+template <int S, int COLL, bool CLOSURE, bool FEW = false>
 static void launch_step(const BatchCase* cases, const int32_t* ic, const int32_t* il,
                         int64_t n_items, int grid, int parity, const ClosureParams* cp,
                         cudaStream_t s) {
   const size_t smem = CLOSURE ? sizeof(ClosureCta) : 0;
-  batch_step_kernel<S, COLL, CLOSURE><<<grid, BT, smem, s>>>(cases, ic, il, n_items, parity, cp);
+  batch_step_kernel<S, COLL, CLOSURE, FEW><<<grid, BT, smem, s>>>(cases, ic, il, n_items, parity, cp);
 }
 
 using StepFn = void (*)(const BatchCase*, const int32_t*, const int32_t*, int64_t, int, int,
@@ -206,7 +209,9 @@ static StepFn step_fn_t(int storage, int collision) {
   }
 }
 
-static StepFn step_fn(int storage, int collision, bool closure) {
+static StepFn step_fn(int storage, int collision, bool closure, bool few) {
+  if (few && !closure && storage == S_F32)
+    return collision == C_BGK ? launch_step<S_F32, C_BGK, false, true> : launch_step<S_F32, C_REG, false, true>;
   return closure ? step_fn_t<true>(storage, collision) : step_fn_t<false>(storage, collision);
 }
 
@@ -366,11 +371,12 @@ lbm_status lbm_batch_create(int n_cases, lbm_grid* const* cases, lbm_batch** out
       first += n;
     }
   }
-  b->fn = step_fn(b->storage, b->collision, false);
-  b->fn_cl = step_fn(b->storage, b->collision, true);
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&b->n_sm, cudaDevAttrMultiProcessorCount, dev);
+  const bool few = b->n_items <= 2 * b->n_sm;
+  b->fn = step_fn(b->storage, b->collision, false, few);
+  b->fn_cl = step_fn(b->storage, b->collision, true, few);
   cudaError_t e = cudaMalloc(&b->cases_d, b->cases_h.size() * sizeof(BatchCase));
   if (e == cudaSuccess) e = cudaMalloc(&b->item_case_d, ic.size() * 4);
   if (e == cudaSuccess) e = cudaMalloc(&b->item_local_d, il.size() * 4);
