@@ -516,12 +516,21 @@ template <> struct Pair16<S_BF16> {
   __device__ static __forceinline__ T2 pack(float a, float b) { return __floats2bfloat162_rn(a, b); }
 };
 
-//
-// Five CTAs per SM: with 48 registers BGK spills 48 bytes, and still the FP16
+// The boundary group inside the launch: one voxel per thread, two CTAs per block.
+// Its long chain of dependent operations decides a step on small grids: with two
+// voxels per thread one after the other the 128 x 64 x 64 FP16 channel took 11.5
+// us a step, 9.7 with a launch of its own, 8.8 like this.  Out of line, so that the
+// interior keeps its registers (8-byte spill otherwise).
+template <int S, int COLL>
+__device__ __noinline__ void pair_boundary(const SparseArgs& a, int64_t slot) {
+  sparse_update<S, 8, COLL, MODE_BOUNDARY>(a, slot);
+}
+
+// Five CTAs per SM: with 48 registers BGK spills 40 bytes, and still the FP16
 // channel takes 174 us a step against 178 at four (REG, no spill: 173 against
 // 184); six spill 212 bytes and take 232.
 template <int S, int COLL, bool GROUP>
-__global__ void __launch_bounds__(SP_THREADS, 5) sparse_pair16(SparseArgs a) {
+__global__ void __launch_bounds__(SP_THREADS, 5) sparse_pair16(const __grid_constant__ SparseArgs a) {
   static_assert(Q == 19 && S != S_F32, "two-voxel kernel: D3Q19, 16-bit storage");
   using T = typename Codec<S>::T;
   using P = Pair16<S>;
@@ -532,9 +541,7 @@ __global__ void __launch_bounds__(SP_THREADS, 5) sparse_pair16(SparseArgs a) {
   chain();
   if constexpr (GROUP) {
     if ((int)blockIdx.x < a.bnd_ctas) {
-      const int64_t slot = (int64_t)blockIdx.x * E3 + t;
-      sparse_update<S, 8, COLL, MODE_BOUNDARY>(a, slot);
-      sparse_update<S, 8, COLL, MODE_BOUNDARY>(a, slot + SP_THREADS);
+      pair_boundary<S, COLL>(a, (int64_t)blockIdx.x * SP_THREADS + t);
       return;
     }
   }
@@ -755,7 +762,7 @@ static void launch_range(Grid& g, SparseArgs a, cudaStream_t s, const char* name
     // 16-bit storage: two voxels per thread, one CTA per block (the range
     // is whole blocks)
     if (i32) {
-      a.bnd_ctas = GROUP ? (int)(a.s0 / E3) : 0;
+      a.bnd_ctas = GROUP ? (int)(a.s0 / SP_THREADS) : 0;
       launch_step(chained, sparse_pair16<S, COLL, GROUP>, (unsigned)((a.s1 - a.s0) / E3) + a.bnd_ctas, SP_THREADS, 0, s, a);
       pair = true;
     }
