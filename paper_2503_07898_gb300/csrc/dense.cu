@@ -59,8 +59,10 @@ __device__ __forceinline__ void boundary_voxel(const DenseArgs& a, int64_t t) {
 // they need neither a second stream nor its two events per step, and a
 // chain of launches overlaps each launch with the one before it (32^3 cavity:
 // 6.5 us a step with a launch per group, 4.5 us; 32^3 periodic 4.4 -> 2.4 us).
+// D3Q27 FP32 with the boundary code spills 124 bytes at four CTAs per SM and none at
+// three (80 x 40 x 40 cavity 11.0 -> 8.5 us; 10.0 with a launch per group).
 template <int S, int COLL, class IDX, bool GROUP>
-__global__ void __launch_bounds__(256, S == S_F32 ? 4 : 5) dense_interior(DenseArgs a, DensePops p,
+__global__ void __launch_bounds__(256, S == S_F32 ? (Q == 27 && GROUP ? 3 : 4) : 5) dense_interior(DenseArgs a, DensePops p,
                                                                           int lid) {
   using T = typename Codec<S>::T;
   int z = blockIdx.z;
@@ -329,8 +331,8 @@ static lbm_status dense_step_t(Grid& g, Level& L, cudaStream_t s) {
     // are recorded; where the boundary code makes the interior spill, only on
     // grids where that costs less than the 3 us of a second stream.  16-bit
     // storage, 48 registers: up to 2 M voxels (256^3 FP16 cavity 266 -> 292 us a
-    // step; D3Q27 at 80^3 20.0 -> 17.3, 128^3 58.8 -> 57.9).  D3Q27 FP32, 64: up
-    // to 64^3 (12.5 -> 10.8 us; at 112^3 52.8 -> 56.1, at 256^3 535 -> 583))
+    // step; D3Q27 at 80^3 20.0 -> 17.3, 128^3 58.8 -> 57.9).  D3Q27 FP32, three
+    // CTAs per SM: up to 64^3 (12.5 -> 10.7 us; at 256^3 535 -> 559))
     constexpr int64_t one_max = S != S_F32 ? (1 << 21) : (Q == 27 ? (1 << 18) : INT64_MAX);
     const bool one = !vec_ok && !g.prof && L.n_reg > 0 && zc > 0 && L.nz < 65535 &&
                      L.n_slots <= one_max &&
