@@ -428,18 +428,19 @@ __device__ __forceinline__ void sparse_update(const SparseArgs& a, int64_t slot)
 //   D3Q19 FP32, 64-bit offsets (496 x 496 x 480): 4 CTAs BGK 3038, REG 3099;
 //     6 spill 190-210 bytes with the boundary group: 3277, 3164
 //   D3Q19 16-bit: 6 with 32-bit offsets, 5 with 64-bit ones
-//   D3Q19 FP32, bitmask grouping (always 64-bit offsets, 40-64 bytes): 6 CTAs
-//     317, 4 321
+//   bitmask grouping, 32-bit offsets (the channel): FP32 D3Q19 285, FP16 219, FP32
+//     D3Q27 428; 64-bit ones for every level had 321, 268 and 474, and at this many
+//     CTAs spilled (small grids up to 20 % slower): they keep 4, 5 and 3
 //   D3Q27 (half-size FP32 REG channel): 3 CTAs 70.5, 4 63.4, 5 with a spill 72.8;
 //     FP32 with 64-bit offsets (440 x 440 x 416, 60-72 bytes at 4): BGK 3 CTAs
 //     3055, 4 3081; REG 3 3104, 4 2980
 template <int S, int COLL, int MODE, class IDX>
 constexpr int sparse_min_ctas() {
-  constexpr bool lean = MODE == MODE_INTERIOR, big = lean && sizeof(IDX) == 8;
-  if (!lean && MODE != MODE_INTERIOR_BM) return 1;
-  if (Q == 27) return S == S_F32 && big && COLL == C_BGK ? 3 : 4;
+  constexpr bool bitmask = MODE == MODE_INTERIOR_BM, big = sizeof(IDX) == 8;
+  if (!bitmask && MODE != MODE_INTERIOR) return 1;
+  if (Q == 27) return big && (bitmask || (S == S_F32 && COLL == C_BGK)) ? 3 : 4;
   if (S == S_F32) return big ? 4 : 6;
-  return lean && !big ? 6 : 5;
+  return big ? 5 : 6;
 }
 
 // GROUP: the first CTAs of an interior launch update the boundary group (the
@@ -745,8 +746,8 @@ static void reg_list_t(Grid& g, Level& L, const void* fin, void* fout, float ome
 }
 
 // i32: the level's Q E^3 n_blocks population elements fit in 31 bits, so the
-// lean kernel indexes with 32-bit offsets (fewer integer instructions per
-// pull); the other modes keep 64-bit indexing.
+// lean kernels (bitmask grouping included) index with 32-bit offsets (fewer
+// integer instructions per pull); the other modes keep 64-bit indexing.
 // chained: a step's only stream, so consecutive launches may overlap.
 template <int S, int E, int COLL, int MODE, bool GROUP = false>
 static void launch_range(Grid& g, SparseArgs a, cudaStream_t s, const char* name, int64_t units,
@@ -770,7 +771,7 @@ static void launch_range(Grid& g, SparseArgs a, cudaStream_t s, const char* name
   if (!pair) {
     a.bnd_ctas = GROUP ? (int)((a.s0 + SP_THREADS - 1) / SP_THREADS) : 0;
     nb += (unsigned)a.bnd_ctas;
-    if (MODE == MODE_INTERIOR && i32)
+    if ((MODE == MODE_INTERIOR || MODE == MODE_INTERIOR_BM) && i32)
       launch_step(chained, sparse_kernel<S, E, COLL, MODE, int32_t, GROUP>, nb, SP_THREADS, 0, s, a);
     else
       launch_step(chained, sparse_kernel<S, E, COLL, MODE, int64_t, GROUP>, nb, SP_THREADS, 0, s, a);
@@ -819,7 +820,7 @@ static lbm_status sparse_step_t(Grid& g, Level& L, cudaStream_t s) {
       a.s1 = L.n_blocks * E3;
       launch_range<S, E, COLL, MODE_BOUNDARY_BM>(g, a, sb, "sparse_boundary_bitmask", L.n_upd_b);
       launch_range<S, E, COLL, MODE_INTERIOR_BM>(g, a, s, "sparse_interior_bitmask",
-                                                 L.n_updated - L.n_upd_b);
+                                                 L.n_updated - L.n_upd_b, fits_i32(L, Q));
     } else {
       a.bc = L.bc_grp_d;
       if (!one) {
