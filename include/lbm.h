@@ -349,7 +349,9 @@ lbm_status lbm_conservation_noalloc(const void* f, int storage, int lattice, int
  * the least-squares eddy viscosity over each coarse voxel's 3^3 neighbourhood,
  * d_tau = -3 sum(tau_sgs_dev : S) / sum(2 rho S : S), clamped to
  * [-(tau_coarse - 1/2) + 1e-3, 1/2].  feats (n_c x 16) and targets (n_c) are
- * device arrays, n_c = voxels / r^3 in coarse x-fastest order.  Synchronises. */
+ * device arrays, n_c = voxels / r^3 in coarse x-fastest order.  The workspace
+ * (31 floats per coarse voxel) is obtained through the grid's allocator and up to
+ * 512 MB stay with the grid; calls on one grid take turns.  Synchronises. */
 lbm_status lbm_closure_dataset(lbm_grid* fine, int r, double tau_coarse, float* feats,
                                float* targets);
 
@@ -362,7 +364,9 @@ lbm_status lbm_closure_dataset(lbm_grid* fine, int r, double tau_coarse, float* 
  * constant and keeps scale 1); theta_io (device, 5313 FP32) holds the initial weights for the
  * standardised problem and receives the trained weights with the
  * standardisation folded in (they take raw features).  loss_out (host, may
- * be NULL) receives the last minibatch loss (standardised).  Synchronises. */
+ * be NULL) receives the last minibatch loss (standardised).  Up to 64 MB of
+ * workspace per device are kept between calls and given back whenever a grid
+ * of that device is destroyed.  Synchronises. */
 lbm_status lbm_closure_train(const float* feats, const float* targets, int64_t n, int steps,
                              int batch, float lr, uint64_t seed, float* theta_io,
                              float* loss_out, void* stream);

@@ -182,7 +182,9 @@ static void free_grid(Grid& g) {
   g.dfree(g.partials_d, g.stream);
   g.dfree(g.sums_d, g.stream);
   g.dfree(g.closure_d, g.stream);
+  g.dfree(g.work_d, g.stream);
   g.closure_d = nullptr;
+  g.work_d = nullptr;
   g.status_d = nullptr;
   g.partials_d = nullptr;
   g.sums_d = nullptr;
@@ -295,10 +297,6 @@ static lbm_status dense_groups(Grid& g, Level& L, const float* bc_values, const 
   L.bc_full_d = nullptr;
   lbm_status st;
   if (L.dense_has_flags) {
-    if (g.spare_used) {
-      LBM_CUDA(cudaMemsetAsync(L.f[L.cur ^ 1], 0, L.pop_bytes, g.stream));
-      g.spare_used = false;
-    }
     if ((st = upload(g, &L.flags_d, fl.data(), (size_t)N))) return st;
   }
   // per-voxel wall mask when walls are not only the box sides, or when the

@@ -1011,16 +1011,22 @@ lbm_status lbm_closure_dataset(lbm_grid* h, int r, double tau_coarse, float* fea
   a.cz_ = L.nz / r;
   a.N = L.n_slots;
   const int64_t nc = (int64_t)a.cx_ * a.cy_ * a.cz_;
-  // Scratch: 31 floats per coarse voxel.  The buffer that the next step
-  // overwrites has room for them when r > 1 and holds nothing that is read
-  // before (every voxel of a grid without flags is written by a step).
+  // Workspace: 31 floats per coarse voxel (260 MB at 256^3, r = 2), kept with the
+  // grid up to 512 MB (550 us a call; 819 with an allocation in each).
+  // (The buffer that the next step overwrites would do for its size, but walls
+  // set later leave solid voxels whose stored values the caller can read.)
   const size_t need = (size_t)nc * (Q + 12) * 4;
-  std::lock_guard<std::mutex> hold(g.spare_mutex);
-  const bool spare = !L.flags_d && need <= L.pop_bytes;
-  DevBuf own(spare ? 0 : need);
-  if (!spare && !own.p) return fail(LBM_ERR_OOM, "device allocation failed");
-  if (spare) g.spare_used = true;
-  a.sbar = spare ? (float*)L.f[L.cur ^ 1] : own.f();
+  constexpr size_t kWorkKeep = (size_t)512 << 20;
+  std::lock_guard<std::mutex> hold(g.work_mutex);
+  if (need <= kWorkKeep && need > g.work_bytes) {
+    g.dfree(g.work_d, g.stream);
+    g.work_d = g.dalloc(need, g.stream);
+    g.work_bytes = g.work_d ? need : 0;
+  }
+  const bool kept = need <= g.work_bytes;
+  DevBuf own(kept ? 0 : need);
+  if (!kept && !own.p) return fail(LBM_ERR_OOM, "device allocation failed");
+  a.sbar = kept ? (float*)g.work_d : own.f();
   a.mom = a.sbar + nc * Q;
   a.num = a.mom + nc * 10;
   a.den = a.num + nc;

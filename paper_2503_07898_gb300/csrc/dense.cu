@@ -393,7 +393,6 @@ static lbm_status dense_step_t(Grid& g, Level& L, cudaStream_t s) {
   }
   LBM_CUDA(cudaGetLastError());
   L.cur ^= 1;
-  g.spare_used = false;
   return LBM_OK;
 }
 

@@ -136,11 +136,11 @@ struct Grid {
   cudaStream_t grp_hi = nullptr;
   cudaEvent_t grp_fork = nullptr, grp_join = nullptr;
 
-  // dense grids without flags: lbm_closure_dataset works in the buffer that the
-  // next step overwrites (one call at a time); spare_used: that buffer holds
-  // such values, to be cleared should walls be set before the next step
-  std::mutex spare_mutex;
-  bool spare_used = false;
+  // workspace of lbm_closure_dataset (one call at a time), kept up to 512 MB until
+  // the grid is destroyed
+  std::mutex work_mutex;
+  void* work_d = nullptr;
+  size_t work_bytes = 0;
 
   // learned closure (multi-resolution levels >= 1)
   void* closure_d = nullptr;     // ClosureParams on the device
