@@ -426,7 +426,11 @@ lbm_status lbm_sync(lbm_grid* g);
 
 /* Per-kernel timing.  lbm_profile(g, 1) clears the records and makes every
  * later kernel launch of this grid record a CUDA event pair on its own
- * stream; lbm_profile(g, 0) stops recording.  lbm_profile_read waits for the
+ * stream; lbm_profile(g, 0) stops recording.  While it is 1, voxel groups that
+ * would share a launch get one each, so that each group has its time; with
+ * lbm_profile(g, 2) a step launches what it launches unprofiled, and a launch
+ * that holds both groups of a grid is recorded as "dense_step" or "sparse_step"
+ * with all updated voxels as its units.  lbm_profile_read waits for the
  * grid's stream and aggregates the records per kernel: launches, summed
  * event time and summed units (updated voxels the launches processed).
  * At most `max` entries are written; *n_out receives the number of kernels. */

@@ -538,7 +538,9 @@ def lbm_batch_closure_load(batch, theta, max_edge):
 
 
 def lbm_profile(grid, enable):
-    _check(load().lbm_profile(grid.ptr, int(bool(enable))), "lbm_profile")
+    """0 off, 1 (or True) a launch and a record per group, 2 the launches of an
+    unprofiled step."""
+    _check(load().lbm_profile(grid.ptr, 2 if enable == 2 else int(bool(enable))), "lbm_profile")
 
 
 def lbm_profile_read(grid):

@@ -858,6 +858,7 @@ lbm_status lbm_profile(lbm_grid* h, int enable) {
     prof_clear(g);
   }
   g.prof = enable != 0;
+  g.prof_split = enable != 2;
   return LBM_OK;
 }
 

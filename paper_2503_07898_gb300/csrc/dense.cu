@@ -334,7 +334,7 @@ static lbm_status dense_step_t(Grid& g, Level& L, cudaStream_t s) {
     // step; D3Q27 at 80^3 20.0 -> 17.3, 128^3 58.8 -> 57.9).  D3Q27 FP32, three
     // CTAs per SM: up to 64^3 (12.5 -> 10.7 us; at 256^3 535 -> 559))
     constexpr int64_t one_max = S != S_F32 ? (1 << 21) : (Q == 27 ? (1 << 18) : INT64_MAX);
-    const bool one = !vec_ok && !g.prof && L.n_reg > 0 && zc > 0 && L.nz < 65535 &&
+    const bool one = !vec_ok && !(g.prof && g.prof_split) && L.n_reg > 0 && zc > 0 && L.nz < 65535 &&
                      L.n_slots <= one_max &&
                      (int64_t)gx * gy * 256 * (65535 - zc) >= L.n_reg;
     const bool fork = L.n_reg > 0 && zc > 0 && !one;
@@ -370,7 +370,8 @@ static lbm_status dense_step_t(Grid& g, Level& L, cudaStream_t s) {
       }
       prof_end(g, s, pr);
     } else if (zc > 0) {
-      const int pr = prof_begin(g, s, "dense_interior", L.n_updated - L.n_reg);
+      const int pr = one ? prof_begin(g, s, "dense_step", L.n_updated)
+                         : prof_begin(g, s, "dense_interior", L.n_updated - L.n_reg);
       using T = typename Codec<S>::T;
       DensePops p;
       for (int i = 0; i < Q; ++i) {

@@ -146,8 +146,9 @@ struct Grid {
   void* closure_d = nullptr;     // ClosureParams on the device
   bool closure_loaded = false;
 
-  // per-kernel event timing (lbm_profile)
-  bool prof = false;
+  // per-kernel event timing (lbm_profile); prof_split: groups that share a launch get
+  // one each while it is on
+  bool prof = false, prof_split = true;
   std::vector<std::string> prof_names;
   std::vector<ProfRec> prof_recs;
 

@@ -805,7 +805,7 @@ static lbm_status sparse_step_t(Grid& g, Level& L, cudaStream_t s) {
     // (one launch holds both groups under the memory grouping, unless their
     // times are recorded)
     const bool both = L.n_b > 0 && L.n_b < L.n_blocks;
-    const bool one = both && !L.bitmask && !g.prof && !(E == 8 && L.variant == VARIANT_STAGED);
+    const bool one = both && !L.bitmask && !(g.prof && g.prof_split) && !(E == 8 && L.variant == VARIANT_STAGED);
     const bool fork = both && !one;
     cudaStream_t sb = s;
     if (fork) {
@@ -838,7 +838,7 @@ static lbm_status sparse_step_t(Grid& g, Level& L, cudaStream_t s) {
         }
       }
       if (one)
-        launch_range<S, E, COLL, MODE_INTERIOR, true>(g, a, s, "sparse_interior", L.n_updated, fits_i32(L, Q), true);
+        launch_range<S, E, COLL, MODE_INTERIOR, true>(g, a, s, "sparse_step", L.n_updated, fits_i32(L, Q), true);
       else if (!staged)
         launch_range<S, E, COLL, MODE_INTERIOR>(g, a, s, "sparse_interior", L.n_updated - L.n_upd_b,
                                                 fits_i32(L, Q), !fork);
