@@ -134,9 +134,9 @@ __global__ void __launch_bounds__(256, 6) k_init_eq(LevelDev d, void* f, const d
 
 // Six CTAs per SM (40 registers) against the five that 48 allow: 256^3, D3Q19
 // FP32 402 -> 369 us, FP16 380 -> 369, D3Q27 FP32 495 -> 429, but D3Q27 FP16
-// 412 -> 443, which keeps five.
+// 412 -> 443, which is left to the compiler.
 template <int S, bool DENSE>
-__global__ void __launch_bounds__(256, Q == 27 && S != S_F32 ? 5 : 6)
+__global__ void __launch_bounds__(256, Q == 27 && S != S_F32 ? 0 : 6)
     k_moments(LevelDev d, const void* f, double* __restrict__ rho, double* __restrict__ u) {
   using T = typename Codec<S>::T;
   const int64_t n = (int64_t)d.nx * d.ny * d.nz;
