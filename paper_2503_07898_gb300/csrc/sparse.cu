@@ -527,11 +527,14 @@ __device__ __noinline__ void pair_boundary(const SparseArgs& a, int64_t slot) {
   sparse_update<S, 8, COLL, MODE_BOUNDARY>(a, slot);
 }
 
-// Five CTAs per SM: with 48 registers BGK spills 40 bytes, and still the FP16
-// channel takes 174 us a step against 178 at four (REG, no spill: 173 against
-// 184); six spill 212 bytes and take 232.
-template <int S, int COLL, bool GROUP>
-__global__ void __launch_bounds__(SP_THREADS, 5) sparse_pair16(const __grid_constant__ SparseArgs a) {
+// CTAS per SM.  Five for chained steps: with 48 registers BGK spills 40 bytes, and
+// still the FP16 channel takes 174 us a step against 178 at four (REG, no spill: 173
+// against 184); six spill 212 bytes and take 232.  Four for launches between others
+// (the levels of a multi-resolution grid), which are often less than a wave, so that
+// the spill counts: three levels in 128 x 128 x 256, FP16 BGK, 8 steps, 1158 -> 1124
+// us (256^3 2501 -> 2478).
+template <int S, int COLL, bool GROUP, int CTAS>
+__global__ void __launch_bounds__(SP_THREADS, CTAS) sparse_pair16(const __grid_constant__ SparseArgs a) {
   static_assert(Q == 19 && S != S_F32, "two-voxel kernel: D3Q19, 16-bit storage");
   using T = typename Codec<S>::T;
   using P = Pair16<S>;
@@ -764,7 +767,8 @@ static void launch_range(Grid& g, SparseArgs a, cudaStream_t s, const char* name
     // is whole blocks)
     if (i32) {
       a.bnd_ctas = GROUP ? (int)(a.s0 / SP_THREADS) : 0;
-      launch_step(chained, sparse_pair16<S, COLL, GROUP>, (unsigned)((a.s1 - a.s0) / E3) + a.bnd_ctas, SP_THREADS, 0, s, a);
+      launch_step(chained, chained ? sparse_pair16<S, COLL, GROUP, 5> : sparse_pair16<S, COLL, GROUP, GROUP ? 5 : 4>,
+                  (unsigned)((a.s1 - a.s0) / E3) + a.bnd_ctas, SP_THREADS, 0, s, a);
       pair = true;
     }
   }
