@@ -46,8 +46,8 @@ METRIC = "D3Q19 GLUPS & % HBM roofline, FP32 vs FP16-store/learned at stated err
 # one 256^3 launch, profiles/f16_kernels_current_ncu.md; keyed by the profiler's
 # name and storage.  FP32: both groups in one launch, 4,096,000 updates to
 # 16,777,216; FP16: the interior group, 4,070,400 to 16,711,680.
-NCU_TRAFFIC = {("dense_step", "f32"): {"bytes_per_launch": 2.353981e+09, "src_sha": "6d7b98ab2a2cee1d"},
-               ("dense_interior", "f16"): {"bytes_per_launch": 1.108861e+09, "src_sha": "6d7b98ab2a2cee1d"}}
+NCU_TRAFFIC = {("dense_step", "f32"): {"bytes_per_launch": 2.354121e+09, "src_sha": "859018c41c9077ef"},
+               ("dense_interior", "f16"): {"bytes_per_launch": 1.108737e+09, "src_sha": "859018c41c9077ef"}}
 
 
 def src_hash():

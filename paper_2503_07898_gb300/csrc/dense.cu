@@ -54,15 +54,24 @@ __device__ __forceinline__ void boundary_voxel(const DenseArgs& a, int64_t t) {
   store_all<S>((T*)a.fout, a, v, g);
 }
 
+// Resident CTAs per SM.  D3Q27 FP32 with the boundary code spills 124 bytes at four
+// and none at three (80 x 40 x 40 cavity 11.0 -> 8.5 us; 10.0 with a launch per
+// group).  16-bit storage with 64-bit offsets (more than 2^31 voxels; measured with
+// them forced on the 256^3 FP16 cavity): D3Q19 BGK 511 us a step at five, 398 at
+// four, 367 at three (332, 140 and 12 bytes of spills); D3Q27 1024, 891, 678.
+template <int S, class IDX, bool GROUP>
+constexpr int dense_ctas() {
+  if (S == S_F32) return Q == 27 && GROUP ? 3 : 4;
+  return sizeof(IDX) == 8 ? 3 : 5;
+}
+
 // GROUP: the first `lid` z slices of CTAs update the boundary group instead.  Both
 // groups read the previous state and write disjoint voxels; in one launch
 // they need neither a second stream nor its two events per step, and a
 // chain of launches overlaps each launch with the one before it (32^3 cavity:
 // 6.5 us a step with a launch per group, 4.5 us; 32^3 periodic 4.4 -> 2.4 us).
-// D3Q27 FP32 with the boundary code spills 124 bytes at four CTAs per SM and none at
-// three (80 x 40 x 40 cavity 11.0 -> 8.5 us; 10.0 with a launch per group).
 template <int S, int COLL, class IDX, bool GROUP>
-__global__ void __launch_bounds__(256, S == S_F32 ? (Q == 27 && GROUP ? 3 : 4) : 5) dense_interior(DenseArgs a, DensePops p,
+__global__ void __launch_bounds__(256, dense_ctas<S, IDX, GROUP>()) dense_interior(DenseArgs a, DensePops p,
                                                                           int lid) {
   using T = typename Codec<S>::T;
   int z = blockIdx.z;
